@@ -333,7 +333,8 @@ def run_native(args):
     # roofline of the dominant kernel (the fused step): algorithmic bytes per launch
     # over the average launch duration seen by events bracketing lbm_step
     step_s = sum(a.elapsed_time(b) for a, b in step_ev) / 1e3
-    launches = sum(w.steps for w in works) * args.steps
+    solve_launches = [lbm.lbm_step_launches(lat.h, w.steps) for w, lat in zip(works, lats)]
+    launches = sum(solve_launches) * args.steps
     per_launch = step_s / launches
     bytes_launch = BYTES_PER_CELL[works[0].storage] * works[0].cells
     peaks = measured_peaks()
@@ -353,7 +354,9 @@ def run_native(args):
             "graph_replayed_copy_method": l2_graph["method"],
             "probe_copy_2x2GB_gbs": hbm_probe["gbs"],
             "l2_traffic": profiled_traffic("l2_bytes_per_launch"),
-            "kernel": STEP_KERNEL[lats[0].cells_per_thread],
+            "kernel": STEP_KERNEL["march" if solve_launches[0] < works[0].steps
+                                  else lats[0].cells_per_thread],
+            "steps_per_launch": works[0].steps / solve_launches[0],
             "cells_per_thread": lats[0].cells_per_thread,
             "bytes_per_launch": bytes_launch, "avg_launch_us": per_launch * 1e6,
             "peak_source": "measured in this run: " + l2["method"],
@@ -397,7 +400,7 @@ def run_native(args):
     if not args.no_e2e:
         e2e = run_e2e(works, lats, stream, dev, args.steps)
 
-    launches_total = args.steps * sum(w.steps + 1 + 4 for w in works)
+    launches_total = args.steps * sum(n + 1 + 4 for n in solve_launches)
     for lat in lats:
         lat.close()
     batched = None
@@ -487,7 +490,9 @@ STEP_KERNEL = {1: "lbm::step_kernel<float, variant, Dirichlet> (one cell per thr
                "tb2": "lbm::step_tb2_kernel<float, variant, Dirichlet> (two cells per thread, "
                       "two time steps per launch through shared memory)",
                "tb2_tma": "lbm::step_tb2_tma_kernel<variant> (two time steps per launch, each "
-                          "tile's input staged by one TMA bulk tensor copy)"}
+                          "tile's input staged by one TMA bulk tensor copy)",
+               "march": "lbm::march_kernel<float, variant, Dirichlet, 3> (warps marching down the "
+                        "lattice, three time steps per launch in registers)"}
 
 
 def timed_steps(w, steps: int, cells=None, per_launch=None, warm: int = 10, tma=None):
@@ -509,7 +514,7 @@ def timed_steps(w, steps: int, cells=None, per_launch=None, warm: int = 10, tma=
             lat.steps_per_launch = per_launch
         if tma is not None:
             lat.tma_staging = tma
-        spl = lat.steps_per_launch
+        spl = steps / lbm.lbm_step_launches(lat.h, steps)
         staged = spl == 2 and lat.tma_staging
         lat.step(warm)
         a = torch.cuda.Event(enable_timing=True)
@@ -524,10 +529,10 @@ def timed_steps(w, steps: int, cells=None, per_launch=None, warm: int = 10, tma=
 
 def roofline_large(peaks, side: int = 4096, steps: int = 100):
     """The FP32 step on a lattice larger than L2 (HBM-bound): the library's
-    default there (two cells per thread, two time steps per launch), and for
-    comparison one step per launch with two cells and with one cell per thread.
+    default there (three time steps per launch in registers), and for comparison
+    two steps per launch through shared memory, one step per launch with two cells and with one cell per thread.
     Algorithmic bytes per launch: 72 B per cell (9 FP32 populations read and
-    written once), whether the launch advances one step or two."""
+    written once), whether the launch advances one step or more."""
     w = wl.quiescent(side, storage="f32", steps=steps, width=128, pulse=True)
     out = {}
     for key, cells, per_launch, tma in (("default", None, None, None),
@@ -540,7 +545,8 @@ def roofline_large(peaks, side: int = 4096, steps: int = 100):
         out[key] = {"steps_per_launch": spl, "avg_launch_us": per_launch_s * 1e6,
                     "mlups": w.cells * steps / t / 1e6,
                     "achieved": achieved, "frac": achieved / peaks["hbm_gbs"],
-                    "kernel": STEP_KERNEL[("tb2_tma" if staged else "tb2") if spl == 2
+                    "kernel": STEP_KERNEL["march" if spl > 2 else
+                                          ("tb2_tma" if staged else "tb2") if spl == 2
                                           else (cells or 2)]}
     d = out["default"]
     # a kernel that moves 72 B per cell and step at the full copy bandwidth

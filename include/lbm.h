@@ -147,10 +147,20 @@ int lbm_init_equilibrium(lbm_handle h, const double* rho, const double* ux, cons
  * half_width <= 0. */
 int lbm_init_pulse(lbm_handle h, double eps, double half_width, double x0, double y0);
 
-/* Advance nsteps >= 0 time steps: one fused kernel per step (pull-stream,
- * moments, rho* and j*, MRT relaxation, damping term, back-transform,
- * store), asynchronous on the handle's stream. */
+/* Advance nsteps >= 0 time steps by fused kernels (pull-stream, moments, rho*
+ * and j*, MRT relaxation, damping term, back-transform, store), asynchronous
+ * on the handle's stream.  Large lattices (about 900 x 900 cells and more)
+ * take groups of two or three steps per launch, by warps that march down the
+ * lattice with the time levels between in registers; the results are those of
+ * the launches that lbm_set_steps_per_launch describes, bit for bit, and
+ * lbm_set_steps_per_launch or lbm_set_tma_staging (or their environment
+ * variables) select those launches instead. */
 int lbm_step(lbm_handle h, int nsteps);
+
+/* Step kernels that lbm_step(h, nsteps) launches as the handle is set up now,
+ * those of replayed graphs included (LBM_ERR_ARG for a NULL handle or
+ * nsteps < 0).  No CUDA call. */
+int lbm_step_launches(lbm_handle h, int nsteps);
 
 /* Fields at the current time: rho_dev = rho - rho0, ux, uy (FP64 [ny][nx];
  * any pointer may be NULL to skip it).  on_device != 0: device pointers,
@@ -187,8 +197,8 @@ int64_t lbm_time(lbm_handle h);
 /* How lbm_step issues its kernels: 0 one launch per step; 1 one launch per
  * step, each a programmatic dependent of the previous (its launch overlaps
  * the previous step's tail); 2 (default) replays of a captured graph of 64
- * steps of such launches (64 one-step or 32 two-step launches), with single
- * launches for the remainder.  All three compute identical results.  The environment variable LBM_LAUNCH=plain|pdl|graph
+ * steps of such launches (64 one-step or 32 two-step launches; 66 steps where
+ * launches take three), with single launches for the remainder.  All three compute identical results.  The environment variable LBM_LAUNCH=plain|pdl|graph
  * sets the initial mode of new handles. */
 int lbm_set_launch_mode(lbm_handle h, int mode);
 
@@ -218,7 +228,10 @@ int lbm_cells_per_thread(lbm_handle h);
  * unsupported 2.  Waits for the handle's stream.  New handles start with 2
  * where it is available and the two population buffers together exceed the
  * device's L2 cache (the step is then HBM-bound), else 1; the environment
- * variable LBM_SPL=1|2 overrides that choice. */
+ * variable LBM_SPL=1|2 overrides that choice.  The value says when 16-bit
+ * states are rounded to the format (every step, or every second); a new handle
+ * may take more steps in one launch with the same results (lbm_step) until
+ * this call names the launches. */
 int lbm_set_steps_per_launch(lbm_handle h, int steps);
 /* The current choice (LBM_ERR_ARG for a NULL handle). */
 int lbm_steps_per_launch(lbm_handle h);
@@ -257,7 +270,9 @@ int lbm_get_arithmetic(lbm_handle h);
  * together exceed four times the L2 size (the environment variable LBM_TMA=0
  * or 1 at lbm_create overrides that choice; 16-bit storage measured level
  * with plain loads and is not staged by default); LBM_ERR_ARG for other
- * handles or values.  A staged copy that has not
+ * handles or values.  It is the staging of the two-step launches where they
+ * are used: for the steps that a new handle's larger launches (lbm_step) leave
+ * over, or for all of them once this call has been made.  A staged copy that has not
  * completed after a bounded wait (2^20 polls of its mbarrier) stops its CTA,
  * which waits for that copy once more with a 16 times longer bound, and makes
  * the next lbm_moments / lbm_diagnostics / lbm_get_state on the host return

@@ -49,10 +49,13 @@ struct lbm_ctx {
     long long* d_time = nullptr;      // channel boundary: device copy of the step counter
     double* d_src_table = nullptr;    // channel boundary: source scales of the next kGraphChunk steps,
                                       // then their FP32 source populations (9 per step)
+    bool march = false;               // with cpt == 2: groups of march_steps() steps go to the marching
+                                      // kernels (chosen by size, until a kernel is asked for by name)
+    int sms = 0;                      // multiprocessors of the device
     bool initialised = false;
     int64_t time = 0;
     int launch_mode = 2;              // kLaunchGraph; LBM_LAUNCH=plain|pdl|graph overrides
-    cudaGraphExec_t graph[2] = {nullptr, nullptr};  // kGraphChunk steps from buffer 0 / 1
+    cudaGraphExec_t graph[2] = {nullptr, nullptr};  // graph_chunk() steps from buffer 0 / 1
     bool tma = false;                 // two-step launches stage their input by TMA (FP32, Dirichlet)
     bool tma_ready = false;           // tmap / tma_grid / tma_err are set up
     CUtensorMap tmap[2];              // tensor maps of buf[0], buf[1]
@@ -69,7 +72,8 @@ namespace {
 // a programmatic dependent of the previous (its launch overlaps the previous
 // step's tail); or replays of a captured graph of kGraphChunk such launches.
 enum { kLaunchPlain = 0, kLaunchPdl = 1, kLaunchGraph = 2 };
-constexpr int kGraphChunk = 64;  // even, so a replay returns to the same buffer
+constexpr int kGraphChunk = 64;  // 64 or 32 launches
+constexpr int kMarchChunk = 66;  // 22 launches of three steps
 
 thread_local std::string g_create_error;
 
@@ -272,6 +276,69 @@ cudaError_t launch_two_steps(lbm_ctx* h, const void* src, void* dst, cudaStream_
     }
 }
 
+// Whether the marching kernels are the faster ones, measured against the one-step
+// pair kernel and the tiles on square lattices (f32, ratio of throughputs):
+//  - Dirichlet: 0.92 at 700^2, 1.00 at 850^2, 1.09 at 900^2, 1.05 at 1024^2, 1.9 at
+//    1300^2, 1.7 at 2048^2, 1.63 at 4096^2 (16-bit storage: 1.03 at 850^2, 1.14-1.17 at
+//    1536^2, 1.3 at 4096^2).  Fewer cells leave too few warps, each with a long walk.
+//  - Periodic, rows a multiple of the staged chunk: 0.94 at 1024^2, 1.14 at 1100^2, 1.8
+//    at 1300^2 and 4096^2 (16-bit: 0.96 at 1024^2, 1.14 at 1300^2, 1.3 at 4096^2).  Other
+//    rows are staged by words at the seam: 0.86 at 1150^2, but 1.12 at 1401^2 and 1.25
+//    at 2049^2 in FP32, once the state exceeds L2.
+//  - At least four strips and 64 rows, or the last strip's idle lanes and the rows
+//    computed twice eat the gain.
+bool march_pays(const lbm_ctx* h, size_t l2) {
+    if (h->nx < 240 || h->ny < 64) return false;
+    const long long cells = static_cast<long long>(h->nx) * h->ny;
+    if (h->bc == LBM_BC_DIRICHLET_EQ) return cells >= 800000;
+    if (h->bc != LBM_BC_PERIODIC) return false;
+    if (h->nx % 4 == 0) return cells >= 1200000;
+    return h->storage == LBM_F32 && 2 * h->buf_bytes > l2;
+}
+
+// Steps of one marching launch.  Results do not depend on it: FP32 levels are
+// what a store would hold, and 16-bit levels are rounded where one (spl = 1) or
+// two steps per launch (spl = 2) round them.
+bool marching(const lbm_ctx* h) { return h->march && h->cpt == 2; }
+int march_steps(const lbm_ctx* h) { return h->storage != LBM_F32 && h->spl == 2 ? 2 : 3; }
+
+cudaError_t launch_march(lbm_ctx* h, const void* src, void* dst, cudaStream_t st, bool pdl) {
+    const int p = pdl ? 1 : 0;
+    const auto* tx = static_cast<const lbm::AxisCoef<float>*>(h->chi_x);
+    const auto* ty = static_cast<const lbm::AxisCoef<float>*>(h->chi_y);
+    const bool periodic = h->bc == LBM_BC_PERIODIC, each = h->spl == 1;
+    switch (h->storage) {
+        case LBM_F32:
+            return (periodic ? lbm::launch_march_f32_periodic : lbm::launch_march_f32_dirichlet)(
+                src, dst, h->geo, h->k2, tx, ty, h->variant, h->sms, st, p);
+        case LBM_F16DEV:
+            return (periodic ? lbm::launch_march_f16_periodic : lbm::launch_march_f16_dirichlet)(
+                src, dst, h->geo, h->k2, tx, ty, h->variant, each, h->sms, st, p);
+        case LBM_BF16DEV:
+            return (periodic ? lbm::launch_march_bf16_periodic : lbm::launch_march_bf16_dirichlet)(
+                src, dst, h->geo, h->k2, tx, ty, h->variant, each, h->sms, st, p);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+// Advance `left` steps' first launch from src to dst; *taken receives its steps.
+cudaError_t launch_steps(lbm_ctx* h, const void* src, void* dst, int left, cudaStream_t st,
+                         bool pdl, long long t_off, int* taken) {
+    if (marching(h) && left >= march_steps(h)) {
+        *taken = march_steps(h);
+        return launch_march(h, src, dst, st, pdl);
+    }
+    *taken = h->spl == 2 && left >= 2 ? 2 : 1;
+    return *taken == 2 ? launch_two_steps(h, src, dst, st, pdl)
+                       : launch_one_step(h, src, dst, st, pdl, t_off);
+}
+
+// Steps of a captured graph: a number of launches that is even, so that a replay
+// returns to the same buffer.
+int graph_chunk(const lbm_ctx* h) {
+    return marching(h) && march_steps(h) == 3 ? kMarchChunk : kGraphChunk;
+}
+
 // Tensor maps, persistent grid and error flag of the TMA two-step kernel;
 // LBM_OK, or the reason it is not available for this handle.
 int setup_tma(lbm_ctx* h) {
@@ -321,7 +388,7 @@ void drop_graphs(lbm_ctx* h) {
     }
 }
 
-// Capture kGraphChunk consecutive steps starting from buffer `parity` on the
+// Capture graph_chunk() consecutive steps starting from buffer `parity` on the
 // handle's private capture stream (programmatic dependent launches between
 // them) and instantiate the graph; it is replayed on the handle's stream.
 cudaError_t ensure_graph(lbm_ctx* h, int parity) {
@@ -335,11 +402,9 @@ cudaError_t ensure_graph(lbm_ctx* h, int parity) {
     if (e != cudaSuccess) return e;
     if (h->bc == LBM_BC_CHANNEL) e = launch_source_table(h, h->capture_stream, kGraphChunk);
     int c = parity;
-    for (int t = 0; t < kGraphChunk && e == cudaSuccess; t += h->spl) {
-        if (h->spl == 2)
-            e = launch_two_steps(h, h->buf[c], h->buf[1 - c], h->capture_stream, t > 0);
-        else
-            e = launch_one_step(h, h->buf[c], h->buf[1 - c], h->capture_stream, t > 0, t);
+    const int chunk = graph_chunk(h);
+    for (int t = 0, n = 0; t < chunk && e == cudaSuccess; t += n) {
+        e = launch_steps(h, h->buf[c], h->buf[1 - c], chunk - t, h->capture_stream, t > 0, t, &n);
         c = 1 - c;
     }
     if (e == cudaSuccess && h->bc == LBM_BC_CHANNEL) {  // the line source's clock
@@ -495,6 +560,10 @@ int lbm_create(int nx, int ny, lbm_storage storage, double rho0, double ux0, dou
     if (tma_env) want_tma = std::strcmp(tma_env, "0") != 0;
     if (storage != LBM_F64 && bc == LBM_BC_DIRICHLET_EQ && want_tma)
         h->tma = setup_tma(h) == LBM_OK;
+    // an environment variable that names a kernel keeps to it
+    h->march = h->cpt == 2 && !std::getenv("LBM_SPL") && !tma_env && march_pays(h, l2) &&
+               cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device) ==
+                   cudaSuccess;
     h->err.clear();
     set_source_shape(h);
     if (const char* m = std::getenv("LBM_LAUNCH")) {
@@ -635,18 +704,19 @@ int lbm_step(lbm_handle h, int nsteps) {
     DeviceGuard dg(h->device);
     cudaError_t e = cudaSuccess;
     const bool pdl = h->launch_mode != kLaunchPlain;
-    if (h->launch_mode == kLaunchGraph && nsteps >= kGraphChunk) {
+    const int graph_steps = graph_chunk(h);
+    if (h->launch_mode == kLaunchGraph && nsteps >= graph_steps) {
         cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
         e = cudaStreamIsCapturing(h->stream, &cs);
         if (e != cudaSuccess) return cuda_fail(h, e, "cudaStreamIsCapturing");
         if (cs == cudaStreamCaptureStatusNone) {
             e = ensure_graph(h, h->cur);
             if (e != cudaSuccess) return cuda_fail(h, e, "lbm_step graph build");
-            while (nsteps >= kGraphChunk) {
+            while (nsteps >= graph_steps) {
                 e = cudaGraphLaunch(h->graph[h->cur], h->stream);
                 if (e != cudaSuccess) return cuda_fail(h, e, "lbm_step graph launch");
-                h->time += kGraphChunk;  // an even number of launches leaves cur unchanged
-                nsteps -= kGraphChunk;
+                h->time += graph_steps;  // an even number of launches leaves cur unchanged
+                nsteps -= graph_steps;
             }
         }
     }
@@ -660,10 +730,9 @@ int lbm_step(lbm_handle h, int nsteps) {
         }
         int issued = 0;
         while (issued < chunk) {
-            const int n = (h->spl == 2 && chunk - issued >= 2) ? 2 : 1;
-            e = n == 2 ? launch_two_steps(h, h->buf[h->cur], h->buf[1 - h->cur], h->stream, pdl)
-                       : launch_one_step(h, h->buf[h->cur], h->buf[1 - h->cur], h->stream, pdl,
-                                         issued);
+            int n = 0;
+            e = launch_steps(h, h->buf[h->cur], h->buf[1 - h->cur], chunk - issued, h->stream, pdl,
+                             issued, &n);
             if (e != cudaSuccess) return cuda_fail(h, e, "lbm_step launch");
             h->cur = 1 - h->cur;
             h->time += n;
@@ -677,6 +746,19 @@ int lbm_step(lbm_handle h, int nsteps) {
         }
     }
     return LBM_OK;
+}
+
+int lbm_step_launches(lbm_handle h, int nsteps) {
+    if (!h) return LBM_ERR_ARG;
+    if (nsteps < 0) return fail(h, LBM_ERR_ARG, "nsteps < 0");
+    const auto launches = [&](int n) {  // of n steps without a graph
+        const int m = marching(h) ? n / march_steps(h) : 0;
+        const int rest = n - m * (m ? march_steps(h) : 0);
+        return m + (h->spl == 2 ? rest / 2 + rest % 2 : rest);
+    };
+    const int chunk = graph_chunk(h);
+    const int graphs = h->launch_mode == kLaunchGraph ? nsteps / chunk : 0;
+    return graphs * launches(chunk) + launches(nsteps - graphs * chunk);
 }
 
 int lbm_moments(lbm_handle h, double* rho_dev, double* ux, double* uy, int on_device) {
@@ -787,10 +869,11 @@ int lbm_set_steps_per_launch(lbm_handle h, int steps) {
         return fail(h, LBM_ERR_ARG, "two steps per launch needs two cells per thread");
     if (steps == 2 && h->bc == LBM_BC_CHANNEL)
         return fail(h, LBM_ERR_ARG, "two steps per launch is not available for the channel boundary");
-    if (steps != h->spl) {
+    if (steps != h->spl || h->march) {
         DeviceGuard dg(h->device);
         cudaStreamSynchronize(h->stream);
         drop_graphs(h);  // the captured launches name the other kernel
+        h->march = false;
         h->spl = steps;
     }
     return LBM_OK;
@@ -822,7 +905,7 @@ int lbm_get_arithmetic(lbm_handle h) { return h ? h->arith : LBM_ERR_ARG; }
 int lbm_set_tma_staging(lbm_handle h, int on) {
     if (!h) return LBM_ERR_ARG;
     if (on != 0 && on != 1) return fail(h, LBM_ERR_ARG, "on must be 0 or 1");
-    if (on == (h->tma ? 1 : 0)) return LBM_OK;
+    if (on == (h->tma ? 1 : 0) && !h->march) return LBM_OK;
     if (on && h->arith == LBM_ARITH_COMPENSATED)
         return fail(h, LBM_ERR_ARG, "compensated arithmetic steps one cell, one step per launch");
     DeviceGuard dg(h->device);
@@ -832,6 +915,7 @@ int lbm_set_tma_staging(lbm_handle h, int on) {
     }
     cudaStreamSynchronize(h->stream);
     drop_graphs(h);  // the captured launches name the other kernel
+    h->march = false;
     h->tma = on == 1;
     return LBM_OK;
 }

@@ -267,6 +267,34 @@ cudaError_t launch_step_tb2_bf16(const void* src, void* dst, const Geometry& g,
                                  const AxisCoef<float>* ty, int variant, int bc, cudaStream_t st,
                                  int pdl);
 
+// Several steps per launch by marching warps (lbm_march.cuh): src holds time t,
+// dst receives t + 3 (FP32, and 16-bit storage with each_level) or t + 2.  sms:
+// multiprocessors of the device.
+cudaError_t launch_march_f32_dirichlet(const void* src, void* dst, const Geometry& g,
+                                   const StepConst<F2>& k, const AxisCoef<float>* tx,
+                                   const AxisCoef<float>* ty, int variant, int sms,
+                                   cudaStream_t st, int pdl);
+cudaError_t launch_march_f32_periodic(const void* src, void* dst, const Geometry& g,
+                                   const StepConst<F2>& k, const AxisCoef<float>* tx,
+                                   const AxisCoef<float>* ty, int variant, int sms,
+                                   cudaStream_t st, int pdl);
+cudaError_t launch_march_f16_dirichlet(const void* src, void* dst, const Geometry& g,
+                                   const StepConst<F2>& k, const AxisCoef<float>* tx,
+                                   const AxisCoef<float>* ty, int variant, bool each_level, int sms,
+                                   cudaStream_t st, int pdl);
+cudaError_t launch_march_f16_periodic(const void* src, void* dst, const Geometry& g,
+                                   const StepConst<F2>& k, const AxisCoef<float>* tx,
+                                   const AxisCoef<float>* ty, int variant, bool each_level, int sms,
+                                   cudaStream_t st, int pdl);
+cudaError_t launch_march_bf16_dirichlet(const void* src, void* dst, const Geometry& g,
+                                   const StepConst<F2>& k, const AxisCoef<float>* tx,
+                                   const AxisCoef<float>* ty, int variant, bool each_level, int sms,
+                                   cudaStream_t st, int pdl);
+cudaError_t launch_march_bf16_periodic(const void* src, void* dst, const Geometry& g,
+                                   const StepConst<F2>& k, const AxisCoef<float>* tx,
+                                   const AxisCoef<float>* ty, int variant, bool each_level, int sms,
+                                   cudaStream_t st, int pdl);
+
 // Two steps per launch with the tile's input staged by TMA (FP32, Dirichlet):
 // src_map describes the buffer holding time t (extent nx x ny x 9 planes,
 // box 72 x 20 x 9 floats); a persistent grid of `grid` CTAs; *err is set when

@@ -1,0 +1,17 @@
+// The marching kernels for BF16 deviation storage, periodic boundary: two steps per
+// launch with the level between them in FP32 (each_level = false), or three steps
+// each rounded to the format as one step per launch rounds it.
+#include "lbm_march.cuh"
+
+namespace lbm {
+
+cudaError_t launch_march_bf16_periodic(const void* src, void* dst, const Geometry& g,
+                                   const StepConst<F2>& k, const AxisCoef<float>* tx,
+                                   const AxisCoef<float>* ty, int variant, bool each_level,
+                                   int sms, cudaStream_t st, int pdl) {
+    if (each_level)
+        return launch_march_t<__nv_bfloat16, kPeriodic, 3, true>(src, dst, g, k, tx, ty, variant, sms, st, pdl);
+    return launch_march_t<__nv_bfloat16, kPeriodic, 2, false>(src, dst, g, k, tx, ty, variant, sms, st, pdl);
+}
+
+}  // namespace lbm

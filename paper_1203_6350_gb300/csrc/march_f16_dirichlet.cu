@@ -1,0 +1,17 @@
+// The marching kernels for FP16 deviation storage, dirichlet boundary: two steps per
+// launch with the level between them in FP32 (each_level = false), or three steps
+// each rounded to the format as one step per launch rounds it.
+#include "lbm_march.cuh"
+
+namespace lbm {
+
+cudaError_t launch_march_f16_dirichlet(const void* src, void* dst, const Geometry& g,
+                                   const StepConst<F2>& k, const AxisCoef<float>* tx,
+                                   const AxisCoef<float>* ty, int variant, bool each_level,
+                                   int sms, cudaStream_t st, int pdl) {
+    if (each_level)
+        return launch_march_t<__half, kDirichlet, 3, true>(src, dst, g, k, tx, ty, variant, sms, st, pdl);
+    return launch_march_t<__half, kDirichlet, 2, false>(src, dst, g, k, tx, ty, variant, sms, st, pdl);
+}
+
+}  // namespace lbm

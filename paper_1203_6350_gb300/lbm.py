@@ -71,6 +71,7 @@ SIGNATURES = [
                                       ctypes.c_double, ctypes.c_double]),
     ("lbm_init_equilibrium", ctypes.c_int, [_vp, _vp, _vp, _vp, ctypes.c_int]),
     ("lbm_step", ctypes.c_int, [_vp, ctypes.c_int]),
+    ("lbm_step_launches", ctypes.c_int, [_vp, ctypes.c_int]),
     ("lbm_moments", ctypes.c_int, [_vp, _vp, _vp, _vp, ctypes.c_int]),
     ("lbm_diagnostics", ctypes.c_int, [_vp, ctypes.c_int, ctypes.c_int, ctypes.c_int,
                                        ctypes.c_int, _vp]),
@@ -223,6 +224,10 @@ def lbm_init_equilibrium(h, rho_ptr, ux_ptr, uy_ptr, on_device) -> int:
 
 def lbm_step(h, nsteps) -> int:
     return load().lbm_step(h, int(nsteps))
+
+
+def lbm_step_launches(h, nsteps) -> int:
+    return load().lbm_step_launches(h, int(nsteps))
 
 
 def lbm_moments(h, rho_ptr, ux_ptr, uy_ptr, on_device) -> int:
