@@ -26,95 +26,149 @@ __device__ __forceinline__ CT feq_dev(int i, CT dr, CT ux, CT uy, CT dux, CT duy
     return weight<CT>(i) * (dr * a + rho0 * b);
 }
 
-template <typename T, int I>
-__device__ __forceinline__ void init_plane(const PlanePtrs<T>& dst, const Geometry& g,
-                                           const BaseState& b, const double* rho, const double* ux,
-                                           const double* uy, int bc, int x, int y) {
+// The base state in the compute precision, converted once on the host (FP64 and the
+// conversions to and from it run at 1/64 of the FP32 rate on GB300, so a kernel that
+// should be bound by memory can afford a few of them per cell, not dozens).
+template <typename CT>
+struct BaseCt {
+    CT rho0, ux0, uy0;
+};
+template <typename T>
+BaseCt<typename Codec<T>::CT> base_ct(const BaseState& b) {
     using CT = typename Codec<T>::CT;
-    // The pull at cell (x, y) + c_I reads this slot, so it holds f^eq there.
-    int sx = x + cx(I), sy = y + cy(I);
-    if (bc == kChannel) sy = (sy + g.ny) % g.ny;  // periodic in y only
-    bool ok = sx >= 0 && sx < g.nx && sy >= 0 && sy < g.ny;
-    if (!ok && bc == kPeriodic) {
-        sx = (sx + g.nx) % g.nx;
-        sy = (sy + g.ny) % g.ny;
-        ok = true;
-    }
-    CT v = CT(0);
-    if (ok) {
-        const long long c = (long long)sy * g.nx + sx;
-        const double u = ux[c], w = uy[c];
-        v = feq_dev<CT>(I, CT(rho[c] - b.rho0), CT(u), CT(w), CT(u - b.ux0), CT(w - b.uy0),
-                        CT(b.rho0), CT(b.ux0), CT(b.uy0));
-    }
-    dst.p[I][(long long)y * g.pitch + x] = Codec<T>::template enc<I>(v);
+    return {CT(b.rho0), CT(b.ux0), CT(b.uy0)};
 }
 
-template <typename T>
-__global__ void init_kernel(PlanePtrs<T> dst, Geometry g, BaseState b, const double* rho,
-                            const double* ux, const double* uy, int bc) {
+template <typename T, int BC, int I>
+__device__ __forceinline__ void put_plane(const PlanePtrs<T>& dst, const Geometry& g, int x, int y,
+                                          typename Codec<T>::CT v, bool interior) {
+    using CT = typename Codec<T>::CT;
+    int tx = x - cx(I), ty = y - cy(I);  // the cell that pulls this population reads slot (tx, ty)
+    if (!interior) {
+        int sx = x + cx(I), sy = y + cy(I);  // the cell whose population this cell's slot holds
+        if (BC != kDirichlet) {  // periodic in y
+            ty = ty < 0 ? g.ny - 1 : ty >= g.ny ? 0 : ty;
+            sy = sy < 0 ? g.ny - 1 : sy >= g.ny ? 0 : sy;
+        }
+        if (BC == kPeriodic) {
+            tx = tx < 0 ? g.nx - 1 : tx >= g.nx ? 0 : tx;
+            sx = sx < 0 ? g.nx - 1 : sx >= g.nx ? 0 : sx;
+        }
+        if (sx < 0 || sx >= g.nx || sy < 0 || sy >= g.ny)
+            dst.p[I][(long long)y * g.pitch + x] = Codec<T>::template enc<I>(CT(0));
+        if (tx < 0 || tx >= g.nx || ty < 0 || ty >= g.ny) return;
+    }
+    dst.p[I][(long long)ty * g.pitch + tx] = Codec<T>::template enc<I>(v);
+}
+
+// Store the equilibrium populations f of cell (x, y) where the first pull reads them,
+// and zero (the far field) in the cell's own slots whose source lies outside the
+// lattice.  Every slot is written once.
+template <typename T, int BC>
+__device__ __forceinline__ void put_cell(const PlanePtrs<T>& dst, const Geometry& g, int x, int y,
+                                         const typename Codec<T>::CT (&f)[9]) {
+    const bool interior = x > 0 && x < g.nx - 1 && y > 0 && y < g.ny - 1;
+    put_plane<T, BC, 0>(dst, g, x, y, f[0], interior);
+    put_plane<T, BC, 1>(dst, g, x, y, f[1], interior);
+    put_plane<T, BC, 2>(dst, g, x, y, f[2], interior);
+    put_plane<T, BC, 3>(dst, g, x, y, f[3], interior);
+    put_plane<T, BC, 4>(dst, g, x, y, f[4], interior);
+    put_plane<T, BC, 5>(dst, g, x, y, f[5], interior);
+    put_plane<T, BC, 6>(dst, g, x, y, f[6], interior);
+    put_plane<T, BC, 7>(dst, g, x, y, f[7], interior);
+    put_plane<T, BC, 8>(dst, g, x, y, f[8], interior);
+}
+
+// Time 0 from FP64 fields.  Each thread takes one cell, converts its three fields
+// once and stores its nine populations; taking each population's source cell instead
+// converted every field nine times.  4096^2 FP32, 24 + 36 B per cell: 2898 us before,
+// 303 us now (3.3 TB/s; the floor at the copy rate is 150 us).
+template <typename T, int BC>
+__global__ void __launch_bounds__(256)
+    init_kernel(PlanePtrs<T> dst, Geometry g, BaseState b, BaseCt<typename Codec<T>::CT> c0,
+                const double* __restrict__ rho, const double* __restrict__ ux,
+                const double* __restrict__ uy) {
+    using CT = typename Codec<T>::CT;
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     if (x >= g.nx || y >= g.ny) return;
-    init_plane<T, 0>(dst, g, b, rho, ux, uy, bc, x, y);
-    init_plane<T, 1>(dst, g, b, rho, ux, uy, bc, x, y);
-    init_plane<T, 2>(dst, g, b, rho, ux, uy, bc, x, y);
-    init_plane<T, 3>(dst, g, b, rho, ux, uy, bc, x, y);
-    init_plane<T, 4>(dst, g, b, rho, ux, uy, bc, x, y);
-    init_plane<T, 5>(dst, g, b, rho, ux, uy, bc, x, y);
-    init_plane<T, 6>(dst, g, b, rho, ux, uy, bc, x, y);
-    init_plane<T, 7>(dst, g, b, rho, ux, uy, bc, x, y);
-    init_plane<T, 8>(dst, g, b, rho, ux, uy, bc, x, y);
+    const long long c = (long long)y * g.nx + x;
+    const double u = ux[c], w = uy[c];
+    const CT dr = CT(rho[c] - b.rho0), cu = CT(u), cw = CT(w);
+    const CT du = b.ux0 == 0.0 ? cu : CT(u - b.ux0), dw = b.uy0 == 0.0 ? cw : CT(w - b.uy0);
+    CT f[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) f[i] = feq_dev<CT>(i, dr, cu, cw, du, dw, c0.rho0, c0.ux0, c0.uy0);
+    put_cell<T, BC>(dst, g, x, y, f);
 }
 
 // Time 0 of the acoustic pulse of Sec. 4.1 (Eqs. pulseprofile, 3:para0) without
 // any input field: rho = rho0 + eps exp(-alpha |x - x_c|^2), u = u0 at every cell.
-template <typename T, int I>
-__device__ __forceinline__ void pulse_plane(const PlanePtrs<T>& dst, const Geometry& g,
-                                            const BaseState& b, double eps, double alpha,
-                                            double xc, double yc, int bc, int x, int y) {
+// A block takes 128 columns and `rows` <= kPulseRows rows.  SEP: the exponential as
+// the product of its two factors, one FP64 exp per column and row of the block and one
+// FP64 product per cell in place of an exp per population; its error of two FP64
+// roundings is far below the FP32 value it is rounded to.  Otherwise (FP64 storage, or
+// alpha not finite) one exp per cell.  4096^2 FP32, 36 B per cell: 8455 us with an exp
+// per population, 184 us now (3.3 TB/s; floor 90 us); 8192^2 BF16 33.8 ms, now 0.45 ms.
+constexpr int kPulseRows = 64;
+template <typename T, int BC, bool SEP>
+__global__ void __launch_bounds__(128)
+    pulse_kernel(PlanePtrs<T> dst, Geometry g, BaseCt<typename Codec<T>::CT> c0, double eps,
+                 double alpha, double xc, double yc, int rows) {
     using CT = typename Codec<T>::CT;
-    int sx = x + cx(I), sy = y + cy(I);
-    if (bc == kChannel) sy = (sy + g.ny) % g.ny;  // periodic in y only
-    bool ok = sx >= 0 && sx < g.nx && sy >= 0 && sy < g.ny;
-    if (!ok && bc == kPeriodic) {
-        sx = (sx + g.nx) % g.nx;
-        sy = (sy + g.ny) % g.ny;
-        ok = true;
+    __shared__ double along_y[SEP ? kPulseRows : 1];
+    const int x = blockIdx.x * 128 + threadIdx.x;
+    const int y0 = blockIdx.y * rows, y1 = min(y0 + rows, g.ny);
+    const double dx = x - xc;
+    double along_x = 0.0;
+    if (SEP) {
+        if (threadIdx.x < rows) {
+            const double dy = static_cast<int>(y0 + threadIdx.x) - yc;
+            along_y[threadIdx.x] = exp(-alpha * (dy * dy));
+        }
+        along_x = eps * exp(-alpha * (dx * dx));
+        __syncthreads();
     }
-    CT v = CT(0);
-    if (ok) {
-        const double dx = sx - xc, dy = sy - yc;
-        const double dr = eps * exp(-alpha * (dx * dx + dy * dy));
-        v = feq_dev<CT>(I, CT(dr), CT(b.ux0), CT(b.uy0), CT(0), CT(0), CT(b.rho0), CT(b.ux0),
-                        CT(b.uy0));
+    if (x >= g.nx) return;
+    for (int y = y0; y < y1; ++y) {
+        double dr;
+        if (SEP) {
+            dr = along_x * along_y[y - y0];
+        } else {
+            const double dy = y - yc;
+            dr = eps * exp(-alpha * (dx * dx + dy * dy));
+        }
+        CT f[9];
+#pragma unroll
+        for (int i = 0; i < 9; ++i)
+            f[i] = feq_dev<CT>(i, CT(dr), c0.ux0, c0.uy0, CT(0), CT(0), c0.rho0, c0.ux0, c0.uy0);
+        put_cell<T, BC>(dst, g, x, y, f);
     }
-    dst.p[I][(long long)y * g.pitch + x] = Codec<T>::template enc<I>(v);
 }
 
-template <typename T>
-__global__ void pulse_kernel(PlanePtrs<T> dst, Geometry g, BaseState b, double eps, double alpha,
-                             double xc, double yc, int bc) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    if (x >= g.nx || y >= g.ny) return;
-    pulse_plane<T, 0>(dst, g, b, eps, alpha, xc, yc, bc, x, y);
-    pulse_plane<T, 1>(dst, g, b, eps, alpha, xc, yc, bc, x, y);
-    pulse_plane<T, 2>(dst, g, b, eps, alpha, xc, yc, bc, x, y);
-    pulse_plane<T, 3>(dst, g, b, eps, alpha, xc, yc, bc, x, y);
-    pulse_plane<T, 4>(dst, g, b, eps, alpha, xc, yc, bc, x, y);
-    pulse_plane<T, 5>(dst, g, b, eps, alpha, xc, yc, bc, x, y);
-    pulse_plane<T, 6>(dst, g, b, eps, alpha, xc, yc, bc, x, y);
-    pulse_plane<T, 7>(dst, g, b, eps, alpha, xc, yc, bc, x, y);
-    pulse_plane<T, 8>(dst, g, b, eps, alpha, xc, yc, bc, x, y);
+template <typename T, int BC>
+cudaError_t pulse_bc(void* dst, const Geometry& g, const BaseState& b, double eps, double alpha,
+                     double xc, double yc, cudaStream_t st) {
+    const PlanePtrs<T> d = plane_ptrs<T>(dst, g.plane);
+    const BaseCt<typename Codec<T>::CT> c0 = base_ct<T>(b);
+    // tall blocks share the exponentials, short ones fill the device on small lattices
+    const int columns = (g.nx + 127) / 128;
+    int rows = kPulseRows;
+    while (rows > 4 && static_cast<long long>(columns) * ((g.ny + rows - 1) / rows) < 608) rows /= 2;
+    const dim3 grid(columns, (g.ny + rows - 1) / rows);
+    if (std::is_same<T, double>::value || !std::isfinite(alpha))
+        pulse_kernel<T, BC, false><<<grid, 128, 0, st>>>(d, g, c0, eps, alpha, xc, yc, rows);
+    else
+        pulse_kernel<T, BC, true><<<grid, 128, 0, st>>>(d, g, c0, eps, alpha, xc, yc, rows);
+    return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t pulse_t(void* dst, const Geometry& g, const BaseState& b, double eps, double alpha,
                     double xc, double yc, int bc, cudaStream_t st) {
-    const dim3 block(128, 2), grid((g.nx + 127) / 128, (g.ny + 1) / 2);
-    pulse_kernel<T><<<grid, block, 0, st>>>(plane_ptrs<T>(dst, g.plane), g, b, eps, alpha, xc, yc, bc);
-    return cudaGetLastError();
+    if (bc == kPeriodic) return pulse_bc<T, kPeriodic>(dst, g, b, eps, alpha, xc, yc, st);
+    if (bc == kChannel) return pulse_bc<T, kChannel>(dst, g, b, eps, alpha, xc, yc, st);
+    return pulse_bc<T, kDirichlet>(dst, g, b, eps, alpha, xc, yc, st);
 }
 
 // rho', j' of the pulled populations at (x, y), summed in the compute precision.
@@ -229,7 +283,14 @@ template <typename T>
 cudaError_t init_t(void* dst, const Geometry& g, const BaseState& b, const double* rho,
                    const double* ux, const double* uy, int bc, cudaStream_t st) {
     const dim3 block(128, 2), grid((g.nx + 127) / 128, (g.ny + 1) / 2);
-    init_kernel<T><<<grid, block, 0, st>>>(plane_ptrs<T>(dst, g.plane), g, b, rho, ux, uy, bc);
+    const PlanePtrs<T> d = plane_ptrs<T>(dst, g.plane);
+    const BaseCt<typename Codec<T>::CT> c0 = base_ct<T>(b);
+    if (bc == kPeriodic)
+        init_kernel<T, kPeriodic><<<grid, block, 0, st>>>(d, g, b, c0, rho, ux, uy);
+    else if (bc == kChannel)
+        init_kernel<T, kChannel><<<grid, block, 0, st>>>(d, g, b, c0, rho, ux, uy);
+    else
+        init_kernel<T, kDirichlet><<<grid, block, 0, st>>>(d, g, b, c0, rho, ux, uy);
     return cudaGetLastError();
 }
 
