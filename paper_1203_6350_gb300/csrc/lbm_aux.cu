@@ -1,6 +1,6 @@
 // Auxiliary kernels: time-0 store at equilibrium, macroscopic fields, and FP64
 // diagnostics reductions.  They read the same pull-stored state as the step.
-#include "d2q9_cell.cuh"
+#include "lbm_read.cuh"
 
 namespace lbm {
 
@@ -190,9 +190,14 @@ __device__ __forceinline__ void cell_moments(const PlanePtrs<T>& src, const Geom
     jy = m[2];
 }
 
+// rho', u of every cell.  States held in FP32 or less: one reciprocal per cell (two FP64
+// instructions) in place of two divisions, and no conversion instructions: eleven FP64
+// instructions per cell, which bound it.  4096^2 FP32, 36 + 24 B per cell: 1143 us
+// with divisions, 472 us now (2.1 TB/s; floor 150 us), the same bits.
 template <typename T, int BC>
-__global__ void moments_kernel(PlanePtrs<T> src, Geometry g, BaseState b, double* rho_dev,
-                               double* ux, double* uy, LineSource ls) {
+__global__ void __launch_bounds__(256)
+    moments_kernel(PlanePtrs<T> src, Geometry g, BaseState b, float rho0_f, double* rho_dev,
+                   double* ux, double* uy, LineSource ls) {
     using CT = typename Codec<T>::CT;
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
@@ -200,83 +205,49 @@ __global__ void moments_kernel(PlanePtrs<T> src, Geometry g, BaseState b, double
     CT r, jx, jy;
     cell_moments<T, BC>(src, g, x, y, r, jx, jy, ls);
     const long long c = (long long)y * g.nx + x;
-    const double rho = b.rho0 + double(r);
-    if (rho_dev) rho_dev[c] = double(r);
-    if (ux) ux[c] = (b.rho0 * b.ux0 + double(jx)) / rho;
-    if (uy) uy[c] = (b.rho0 * b.uy0 + double(jy)) / rho;
-}
-
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    return v;
+    const double dr = widen(r);
+    if (rho_dev) rho_dev[c] = dr;
+    const double rho = b.rho0 + dr;
+    if constexpr (std::is_same<CT, double>::value) {
+        if (ux) ux[c] = __fma_rn(b.rho0, b.ux0, jx) / rho;
+        if (uy) uy[c] = __fma_rn(b.rho0, b.uy0, jy) / rho;
+    } else {
+        const Reciprocal inv = reciprocal(rho, rho0_f + r);
+        if (ux) ux[c] = quotient(__fma_rn(b.rho0, b.ux0, widen(jx)), inv, isfinite(jx));
+        if (uy) uy[c] = quotient(__fma_rn(b.rho0, b.uy0, widen(jy)), inv, isfinite(jy));
+    }
 }
 
 constexpr int kDiagThreads = 256;
 
 // First pass: block (bx, by) of a gx x gy grid takes the rows y0 + by, + gy, ...
 // and the columns x0 + bx * 256 + t, + gx * 256, ... of the region, and writes
-// its kDiag sums (FP64) to partial[by * gx + bx].
+// its kDiag sums (FP64) to partial[by * gx + bx].  4096^2
+// FP32, 36 B per cell: 1020 us with eleven FP64 operations and nine conversions per
+// cell, 414 us now (floor 90 us).
 template <typename T, int BC>
 __global__ void __launch_bounds__(kDiagThreads)
     diag_partial_kernel(PlanePtrs<T> src, Geometry g, BaseState b, int x0, int y0, int x1, int y1,
                         double* partial, LineSource ls) {
     using CT = typename Codec<T>::CT;
-    double acc[kDiag] = {0, 0, 0, 0, 0, 0};
+    DiagSums sums;
     const CT rho0 = CT(b.rho0), ux0 = CT(b.ux0), uy0 = CT(b.uy0);
     for (int y = y0 + blockIdx.y; y < y1; y += gridDim.y) {
         for (int x = x0 + blockIdx.x * kDiagThreads + threadIdx.x; x < x1;
              x += gridDim.x * kDiagThreads) {
             CT r, jx, jy;
             cell_moments<T, BC>(src, g, x, y, r, jx, jy, ls);
-            // u - u0 = (j' - rho' u0) / rho, with j' = j - rho0 u0
-            const CT inv = CT(1) / (rho0 + r);
-            const CT dux = (jx - r * ux0) * inv;
-            const CT duy = (jy - r * uy0) * inv;
-            const double dr = double(r);
-            const double e = dr * dr / (6.0 * b.rho0) +
-                             0.5 * b.rho0 * (double(dux) * double(dux) + double(duy) * double(duy));
-            const bool finite = isfinite(r) && isfinite(dux) && isfinite(duy);
-            acc[0] += dr;
-            acc[1] += double(jx);
-            acc[2] += double(jy);
-            acc[3] += e;
-            acc[4] += dr * dr;
-            acc[5] += finite ? 0.0 : 1.0;
+            sums.add(r, jx, jy, rho0, ux0, uy0);
         }
     }
-    __shared__ double red[kDiag][kDiagThreads / 32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int q = 0; q < kDiag; ++q) {
-        const double v = warp_sum(acc[q]);
-        if (lane == 0) red[q][warp] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < kDiag) {
-        double s = 0.0;
-        for (int k = 0; k < kDiagThreads / 32; ++k) s += red[threadIdx.x][k];
-        partial[(blockIdx.y * gridDim.x + blockIdx.x) * kDiag + threadIdx.x] = s;
-    }
+    write_diag_partial<kDiagThreads>(sums, b.rho0,
+                                     partial + (blockIdx.y * gridDim.x + blockIdx.x) * kDiag);
 }
 
 // Second pass: one block adds the partials in a fixed order.
 __global__ void __launch_bounds__(kDiagThreads)
     diag_final_kernel(const double* partial, int blocks, double* out) {
-    __shared__ double red[kDiag][kDiagThreads / 32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int q = 0; q < kDiag; ++q) {
-        double s = 0.0;
-        for (int k = threadIdx.x; k < blocks; k += kDiagThreads) s += partial[k * kDiag + q];
-        s = warp_sum(s);
-        if (lane == 0) red[q][warp] = s;
-    }
-    __syncthreads();
-    if (threadIdx.x < kDiag) {
-        double s = 0.0;
-        for (int k = 0; k < kDiagThreads / 32; ++k) s += red[threadIdx.x][k];
-        out[threadIdx.x] = s;
-    }
+    sum_diag_partials<kDiagThreads>(partial, blocks, out);
 }
 
 template <typename T>
@@ -299,12 +270,13 @@ cudaError_t moments_t(const void* src, const Geometry& g, const BaseState& b, in
                       double* ux, double* uy, cudaStream_t st, const LineSource& ls) {
     const dim3 block(128, 2), grid((g.nx + 127) / 128, (g.ny + 1) / 2);
     const PlanePtrs<T> s = plane_ptrs<T>(const_cast<void*>(src), g.plane);
+    const float rho0_f = static_cast<float>(b.rho0);
     if (bc == kPeriodic)
-        moments_kernel<T, kPeriodic><<<grid, block, 0, st>>>(s, g, b, r, ux, uy, ls);
+        moments_kernel<T, kPeriodic><<<grid, block, 0, st>>>(s, g, b, rho0_f, r, ux, uy, ls);
     else if (bc == kChannel)
-        moments_kernel<T, kChannel><<<grid, block, 0, st>>>(s, g, b, r, ux, uy, ls);
+        moments_kernel<T, kChannel><<<grid, block, 0, st>>>(s, g, b, rho0_f, r, ux, uy, ls);
     else
-        moments_kernel<T, kDirichlet><<<grid, block, 0, st>>>(s, g, b, r, ux, uy, ls);
+        moments_kernel<T, kDirichlet><<<grid, block, 0, st>>>(s, g, b, rho0_f, r, ux, uy, ls);
     return cudaGetLastError();
 }
 

@@ -3,7 +3,7 @@
 // device array instead of memory the library allocates per call or per handle.
 #include <mutex>
 
-#include "d2q9_cell.cuh"
+#include "lbm_read.cuh"
 #include "lbm.h"
 
 namespace {
@@ -44,12 +44,6 @@ cudaError_t scratch_address(double** out) {
     return cudaSuccess;
 }
 
-__device__ __forceinline__ double na_warp_sum(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    return v;
-}
-
 // Block b sums the cells b * kNaCellsPerBlock ... of the region taken in
 // row-major order (region width w, first cell (x0, y0)).
 template <typename T, int BC>
@@ -57,7 +51,7 @@ __global__ void __launch_bounds__(kNaThreads)
     na_partial_kernel(PlanePtrs<T> src, Geometry g, BaseState b, int x0, int y0, int w,
                       long long ncell, double* partial) {
     using CT = typename Codec<T>::CT;
-    double acc[kDiag] = {0, 0, 0, 0, 0, 0};
+    DiagSums sums;
     const CT rho0 = CT(b.rho0), ux0 = CT(b.ux0), uy0 = CT(b.uy0);
     const long long begin = (long long)blockIdx.x * kNaCellsPerBlock;
     const long long end = begin + kNaCellsPerBlock < ncell ? begin + kNaCellsPerBlock : ncell;
@@ -75,18 +69,7 @@ __global__ void __launch_bounds__(kNaThreads)
         pull_all<T, BC, true>(src, y * pitch + x, ps, v);
         CT m[9];
         moments9(v, m);
-        const CT r = m[0], jx = m[1], jy = m[2];
-        const CT inv = CT(1) / (rho0 + r);
-        const CT dux = (jx - r * ux0) * inv;  // u - u0 = (j' - rho' u0) / rho
-        const CT duy = (jy - r * uy0) * inv;
-        const double dr = double(r);
-        acc[0] += dr;
-        acc[1] += double(jx);
-        acc[2] += double(jy);
-        acc[3] += dr * dr / (6.0 * b.rho0) +
-                  0.5 * b.rho0 * (double(dux) * double(dux) + double(duy) * double(duy));
-        acc[4] += dr * dr;
-        acc[5] += (isfinite(r) && isfinite(dux) && isfinite(duy)) ? 0.0 : 1.0;
+        sums.add(m[0], m[1], m[2], rho0, ux0, uy0);
         rx += step_x;
         ry += step_y;
         if (rx >= w) {
@@ -94,38 +77,13 @@ __global__ void __launch_bounds__(kNaThreads)
             ++ry;
         }
     }
-    __shared__ double red[kDiag][kNaThreads / 32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int q = 0; q < kDiag; ++q) {
-        const double v = na_warp_sum(acc[q]);
-        if (lane == 0) red[q][warp] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < kDiag) {
-        double s = 0.0;
-        for (int k = 0; k < kNaThreads / 32; ++k) s += red[threadIdx.x][k];
-        partial[blockIdx.x * kDiag + threadIdx.x] = s;
-    }
+    write_diag_partial<kNaThreads>(sums, b.rho0, partial + blockIdx.x * kDiag);
 }
 
 // One block adds the partial rows in a fixed order.
 __global__ void __launch_bounds__(kNaThreads)
     na_final_kernel(const double* partial, int blocks, double* out) {
-    __shared__ double red[kDiag][kNaThreads / 32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int q = 0; q < kDiag; ++q) {
-        double s = 0.0;
-        for (int k = threadIdx.x; k < blocks; k += kNaThreads) s += partial[k * kDiag + q];
-        s = na_warp_sum(s);
-        if (lane == 0) red[q][warp] = s;
-    }
-    __syncthreads();
-    if (threadIdx.x < kDiag) {
-        double s = 0.0;
-        for (int k = 0; k < kNaThreads / 32; ++k) s += red[threadIdx.x][k];
-        out[threadIdx.x] = s;
-    }
+    sum_diag_partials<kNaThreads>(partial, blocks, out);
 }
 
 template <typename T>
