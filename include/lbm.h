@@ -151,7 +151,8 @@ int lbm_init_pulse(lbm_handle h, double eps, double half_width, double x0, doubl
  * and j*, MRT relaxation, damping term, back-transform, store), asynchronous
  * on the handle's stream.  Large lattices (about 900 x 900 cells and more)
  * take groups of two or three steps per launch, by warps that march down the
- * lattice with the time levels between in registers; the results are those of
+ * lattice with the time levels between in registers, and small ones (up to
+ * 226 x 226 cells) up to six, on tiles in shared memory; the results are those of
  * the launches that lbm_set_steps_per_launch describes, bit for bit, and
  * lbm_set_steps_per_launch or lbm_set_tma_staging (or their environment
  * variables) select those launches instead. */
@@ -197,8 +198,8 @@ int64_t lbm_time(lbm_handle h);
 /* How lbm_step issues its kernels: 0 one launch per step; 1 one launch per
  * step, each a programmatic dependent of the previous (its launch overlaps
  * the previous step's tail); 2 (default) replays of a captured graph of 64
- * steps of such launches (64 one-step or 32 two-step launches; 66 steps where
- * launches take three), with single launches for the remainder.  All three compute identical results.  The environment variable LBM_LAUNCH=plain|pdl|graph
+ * steps of such launches (64 one-step or 32 two-step launches; 66 or 60 steps
+ * where launches take three or six), with single launches for the remainder.  All three compute identical results.  The environment variable LBM_LAUNCH=plain|pdl|graph
  * sets the initial mode of new handles. */
 int lbm_set_launch_mode(lbm_handle h, int mode);
 

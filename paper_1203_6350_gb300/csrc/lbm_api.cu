@@ -52,6 +52,8 @@ struct lbm_ctx {
     bool march = false;               // with cpt == 2: groups of march_steps() steps go to the marching
                                       // kernels (chosen by size, until a kernel is asked for by name)
     int sms = 0;                      // multiprocessors of the device
+    int tile_h = 0;                   // with cpt == 2: rows of the small-lattice tiles (0: not used),
+    int tile_levels = 0;              // and the steps one of their launches takes at most
     bool initialised = false;
     int64_t time = 0;
     int launch_mode = 2;              // kLaunchGraph; LBM_LAUNCH=plain|pdl|graph overrides
@@ -72,7 +74,7 @@ namespace {
 // a programmatic dependent of the previous (its launch overlaps the previous
 // step's tail); or replays of a captured graph of kGraphChunk such launches.
 enum { kLaunchPlain = 0, kLaunchPdl = 1, kLaunchGraph = 2 };
-constexpr int kGraphChunk = 64;  // 64 or 32 launches
+constexpr int kGraphChunk = 64;  // 64, 32 or 16 launches
 constexpr int kMarchChunk = 66;  // 22 launches of three steps
 
 thread_local std::string g_create_error;
@@ -299,6 +301,54 @@ bool march_pays(const lbm_ctx* h, size_t l2) {
 // Steps of one marching launch.  Results do not depend on it: FP32 levels are
 // what a store would hold, and 16-bit levels are rounded where one (spl = 1) or
 // two steps per launch (spl = 2) round them.
+// Small lattices take several steps per launch on tiles of 32-column regions.  Up to
+// 128^2 cells six steps on tiles of 4 rows (64^2 0.87 us per step, 100^2 0.89; with 8
+// steps 0.90, 0.93); up to 226^2 four steps on tiles of 16 rows (200^2 1.31 us; with six
+// and 10 rows 1.87).  Above, a launch per step is level or faster (300^2 1.97 us
+// against 2.37, 800 x 200 channel 2.63 against 3.3): the cells computed twice fill the GPU.
+constexpr int kTileRegion = 32;
+void choose_tiles(lbm_ctx* h) {
+    const long long cells = static_cast<long long>(h->nx) * h->ny;
+    if (cells <= 128 * 128) {
+        h->tile_h = 4;
+        h->tile_levels = 6;
+    } else if (cells <= 226 * 226) {
+        h->tile_h = 16;
+        h->tile_levels = 4;
+    }
+}
+bool tiled(const lbm_ctx* h) { return h->tile_h > 0 && h->cpt == 2; }
+// Steps of the next launch of `left` >= 2: equal parts of at most tile_levels.
+int tile_steps(const lbm_ctx* h, int left) {
+    const int launches = (left + h->tile_levels - 1) / h->tile_levels;
+    return (left + launches - 1) / launches;
+}
+
+cudaError_t launch_tile(lbm_ctx* h, const void* src, void* dst, int levels, cudaStream_t st,
+                        bool pdl, long long t_off) {
+    const int p = pdl ? 1 : 0;
+    const lbm::LineSource ls = launch_source(h, t_off);
+    const auto* tx = static_cast<const lbm::AxisCoef<float>*>(h->chi_x);
+    const auto* ty = static_cast<const lbm::AxisCoef<float>*>(h->chi_y);
+    const auto launch = h->storage == LBM_F32      ? lbm::launch_tile_f32
+                        : h->storage == LBM_F16DEV ? lbm::launch_tile_f16
+                                                   : lbm::launch_tile_bf16;
+    return launch(src, dst, h->geo, h->k2, tx, ty, h->variant, h->bc, kTileRegion, h->tile_h,
+                  levels, st, p, ls);
+}
+
+// Set the handle's tile kernel up for its variant; without it, no tiles.
+void prepare_tiles(lbm_ctx* h) {
+    if (!h->tile_h) return;
+    const auto prepare = h->storage == LBM_F32      ? lbm::prepare_tile_f32
+                         : h->storage == LBM_F16DEV ? lbm::prepare_tile_f16
+                                                    : lbm::prepare_tile_bf16;
+    if (prepare(h->variant, h->bc, kTileRegion, h->tile_h, h->tile_levels) != cudaSuccess) {
+        cudaGetLastError();
+        h->tile_h = 0;
+    }
+}
+
 bool marching(const lbm_ctx* h) { return h->march && h->cpt == 2; }
 int march_steps(const lbm_ctx* h) { return h->storage != LBM_F32 && h->spl == 2 ? 2 : 3; }
 
@@ -328,6 +378,10 @@ cudaError_t launch_steps(lbm_ctx* h, const void* src, void* dst, int left, cudaS
         *taken = march_steps(h);
         return launch_march(h, src, dst, st, pdl);
     }
+    if (tiled(h) && left >= 2) {
+        *taken = tile_steps(h, left);
+        return launch_tile(h, src, dst, *taken, st, pdl, t_off);
+    }
     *taken = h->spl == 2 && left >= 2 ? 2 : 1;
     return *taken == 2 ? launch_two_steps(h, src, dst, st, pdl)
                        : launch_one_step(h, src, dst, st, pdl, t_off);
@@ -336,6 +390,7 @@ cudaError_t launch_steps(lbm_ctx* h, const void* src, void* dst, int left, cudaS
 // Steps of a captured graph: a number of launches that is even, so that a replay
 // returns to the same buffer.
 int graph_chunk(const lbm_ctx* h) {
+    if (tiled(h)) return h->tile_levels == 6 ? 60 : kGraphChunk;  // 10 or 16 launches
     return marching(h) && march_steps(h) == 3 ? kMarchChunk : kGraphChunk;
 }
 
@@ -400,15 +455,15 @@ cudaError_t ensure_graph(lbm_ctx* h, int parity) {
     }
     e = cudaStreamBeginCapture(h->capture_stream, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return e;
-    if (h->bc == LBM_BC_CHANNEL) e = launch_source_table(h, h->capture_stream, kGraphChunk);
-    int c = parity;
     const int chunk = graph_chunk(h);
+    if (h->bc == LBM_BC_CHANNEL) e = launch_source_table(h, h->capture_stream, chunk);
+    int c = parity;
     for (int t = 0, n = 0; t < chunk && e == cudaSuccess; t += n) {
         e = launch_steps(h, h->buf[c], h->buf[1 - c], chunk - t, h->capture_stream, t > 0, t, &n);
         c = 1 - c;
     }
     if (e == cudaSuccess && h->bc == LBM_BC_CHANNEL) {  // the line source's clock
-        advance_time_kernel<<<1, 1, 0, h->capture_stream>>>(h->d_time, kGraphChunk);
+        advance_time_kernel<<<1, 1, 0, h->capture_stream>>>(h->d_time, chunk);
         e = cudaGetLastError();
     }
     cudaGraph_t g = nullptr;
@@ -564,6 +619,8 @@ int lbm_create(int nx, int ny, lbm_storage storage, double rho0, double ux0, dou
     h->march = h->cpt == 2 && !std::getenv("LBM_SPL") && !tma_env && march_pays(h, l2) &&
                cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device) ==
                    cudaSuccess;
+    if (h->cpt == 2 && h->spl == 1 && !std::getenv("LBM_SPL") && !tma_env) choose_tiles(h);
+    prepare_tiles(h);
     h->err.clear();
     set_source_shape(h);
     if (const char* m = std::getenv("LBM_LAUNCH")) {
@@ -640,6 +697,7 @@ int lbm_set_sponge(lbm_handle h, lbm_variant variant, const double* chi_x, const
     lbm::zero_run(chi_x, h->nx, h->bulk[0], h->bulk[1]);
     lbm::zero_run(chi_y, h->ny, h->bulk[2], h->bulk[3]);
     refresh_consts(h);
+    prepare_tiles(h);
     const double s_nu = h->rates.s[7];
     if ((variant == LBM_SPONGE_II || variant == LBM_SPONGE_III) && chi_max > 4.0 / s_nu)
         return fail(h, LBM_WARN_UNSTABLE_PARAMS, "max chi exceeds the critical value 4/s");
@@ -752,6 +810,7 @@ int lbm_step_launches(lbm_handle h, int nsteps) {
     if (!h) return LBM_ERR_ARG;
     if (nsteps < 0) return fail(h, LBM_ERR_ARG, "nsteps < 0");
     const auto launches = [&](int n) {  // of n steps without a graph
+        if (tiled(h)) return (n + h->tile_levels - 1) / h->tile_levels;
         const int m = marching(h) ? n / march_steps(h) : 0;
         const int rest = n - m * (m ? march_steps(h) : 0);
         return m + (h->spl == 2 ? rest / 2 + rest % 2 : rest);
@@ -869,11 +928,12 @@ int lbm_set_steps_per_launch(lbm_handle h, int steps) {
         return fail(h, LBM_ERR_ARG, "two steps per launch needs two cells per thread");
     if (steps == 2 && h->bc == LBM_BC_CHANNEL)
         return fail(h, LBM_ERR_ARG, "two steps per launch is not available for the channel boundary");
-    if (steps != h->spl || h->march) {
+    if (steps != h->spl || h->march || h->tile_h) {
         DeviceGuard dg(h->device);
         cudaStreamSynchronize(h->stream);
         drop_graphs(h);  // the captured launches name the other kernel
         h->march = false;
+        h->tile_h = 0;
         h->spl = steps;
     }
     return LBM_OK;
@@ -905,7 +965,7 @@ int lbm_get_arithmetic(lbm_handle h) { return h ? h->arith : LBM_ERR_ARG; }
 int lbm_set_tma_staging(lbm_handle h, int on) {
     if (!h) return LBM_ERR_ARG;
     if (on != 0 && on != 1) return fail(h, LBM_ERR_ARG, "on must be 0 or 1");
-    if (on == (h->tma ? 1 : 0) && !h->march) return LBM_OK;
+    if (on == (h->tma ? 1 : 0) && !h->march && !h->tile_h) return LBM_OK;
     if (on && h->arith == LBM_ARITH_COMPENSATED)
         return fail(h, LBM_ERR_ARG, "compensated arithmetic steps one cell, one step per launch");
     DeviceGuard dg(h->device);
@@ -916,6 +976,7 @@ int lbm_set_tma_staging(lbm_handle h, int on) {
     cudaStreamSynchronize(h->stream);
     drop_graphs(h);  // the captured launches name the other kernel
     h->march = false;
+    h->tile_h = 0;
     h->tma = on == 1;
     return LBM_OK;
 }

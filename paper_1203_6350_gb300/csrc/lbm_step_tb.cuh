@@ -53,28 +53,30 @@ __device__ __forceinline__ int wrap_coord(int c, int n) {
 }
 
 // Pull the nine populations of the cells (ca, y) and (cb, y), both inside the
-// lattice, with the boundary rule for their sources.
+// lattice, with the boundary rule for their sources (src_pop: the channel's source
+// populations).
 template <typename T, int BC>
 __device__ __forceinline__ void pull_lanes(const T* __restrict__ s, unsigned plane, int pitch,
-                                           int ca, int cb, int y, int nx, int ny, F2 (&v)[9]) {
-    v[0] = f2(pull_one<T, BC, 0>(s, plane, pitch, ca, y, nx, ny),
-              pull_one<T, BC, 0>(s, plane, pitch, cb, y, nx, ny));
-    v[1] = f2(pull_one<T, BC, 1>(s, plane, pitch, ca, y, nx, ny),
-              pull_one<T, BC, 1>(s, plane, pitch, cb, y, nx, ny));
-    v[2] = f2(pull_one<T, BC, 2>(s, plane, pitch, ca, y, nx, ny),
-              pull_one<T, BC, 2>(s, plane, pitch, cb, y, nx, ny));
-    v[3] = f2(pull_one<T, BC, 3>(s, plane, pitch, ca, y, nx, ny),
-              pull_one<T, BC, 3>(s, plane, pitch, cb, y, nx, ny));
-    v[4] = f2(pull_one<T, BC, 4>(s, plane, pitch, ca, y, nx, ny),
-              pull_one<T, BC, 4>(s, plane, pitch, cb, y, nx, ny));
-    v[5] = f2(pull_one<T, BC, 5>(s, plane, pitch, ca, y, nx, ny),
-              pull_one<T, BC, 5>(s, plane, pitch, cb, y, nx, ny));
-    v[6] = f2(pull_one<T, BC, 6>(s, plane, pitch, ca, y, nx, ny),
-              pull_one<T, BC, 6>(s, plane, pitch, cb, y, nx, ny));
-    v[7] = f2(pull_one<T, BC, 7>(s, plane, pitch, ca, y, nx, ny),
-              pull_one<T, BC, 7>(s, plane, pitch, cb, y, nx, ny));
-    v[8] = f2(pull_one<T, BC, 8>(s, plane, pitch, ca, y, nx, ny),
-              pull_one<T, BC, 8>(s, plane, pitch, cb, y, nx, ny));
+                                           int ca, int cb, int y, int nx, int ny, F2 (&v)[9],
+                                           const float* src_pop = nullptr) {
+    v[0] = f2(pull_one<T, BC, 0>(s, plane, pitch, ca, y, nx, ny, src_pop),
+              pull_one<T, BC, 0>(s, plane, pitch, cb, y, nx, ny, src_pop));
+    v[1] = f2(pull_one<T, BC, 1>(s, plane, pitch, ca, y, nx, ny, src_pop),
+              pull_one<T, BC, 1>(s, plane, pitch, cb, y, nx, ny, src_pop));
+    v[2] = f2(pull_one<T, BC, 2>(s, plane, pitch, ca, y, nx, ny, src_pop),
+              pull_one<T, BC, 2>(s, plane, pitch, cb, y, nx, ny, src_pop));
+    v[3] = f2(pull_one<T, BC, 3>(s, plane, pitch, ca, y, nx, ny, src_pop),
+              pull_one<T, BC, 3>(s, plane, pitch, cb, y, nx, ny, src_pop));
+    v[4] = f2(pull_one<T, BC, 4>(s, plane, pitch, ca, y, nx, ny, src_pop),
+              pull_one<T, BC, 4>(s, plane, pitch, cb, y, nx, ny, src_pop));
+    v[5] = f2(pull_one<T, BC, 5>(s, plane, pitch, ca, y, nx, ny, src_pop),
+              pull_one<T, BC, 5>(s, plane, pitch, cb, y, nx, ny, src_pop));
+    v[6] = f2(pull_one<T, BC, 6>(s, plane, pitch, ca, y, nx, ny, src_pop),
+              pull_one<T, BC, 6>(s, plane, pitch, cb, y, nx, ny, src_pop));
+    v[7] = f2(pull_one<T, BC, 7>(s, plane, pitch, ca, y, nx, ny, src_pop),
+              pull_one<T, BC, 7>(s, plane, pitch, cb, y, nx, ny, src_pop));
+    v[8] = f2(pull_one<T, BC, 8>(s, plane, pitch, ca, y, nx, ny, src_pop),
+              pull_one<T, BC, 8>(s, plane, pitch, cb, y, nx, ny, src_pop));
 }
 
 // Two steps on the tile at (x0, y0) by a block of NT threads (any shape,
