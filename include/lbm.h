@@ -379,6 +379,11 @@ int lbm_batch_cells_per_thread(lbm_batch b);
  * An instance whose budget ends after the first step of a two-step launch
  * takes that one step.  Needs two cells per thread
  * (lbm_batch_set_cells_per_thread(b, 1) switches it back to 1).  Default 1.
+ * With 2, batches of Dirichlet instances of some size (36,000 cells on average,
+ * 16,000 with 16-bit storage) take two (FP32: three) steps per launch by the
+ * marching kernels of lbm_step, with the same results, as long as every active
+ * instance has that many left; the environment variable LBM_BATCH_TMA (either
+ * value) keeps to the tiles.
  * LBM_ERR_ARG for any other value or an unsupported 2.  Waits for the
  * batch's stream. */
 int lbm_batch_set_steps_per_launch(lbm_batch b, int steps);

@@ -10,6 +10,7 @@
 #include "lbm.h"
 #include "lbm_host.h"
 #include "lbm_internal.h"
+#include "lbm_march_cut.h"
 
 using lbm::Geometry;
 using lbm::StepConst;
@@ -51,6 +52,7 @@ struct lbm_ctx {
                                       // then their FP32 source populations (9 per step)
     bool march = false;               // with cpt == 2: groups of march_steps() steps go to the marching
                                       // kernels (chosen by size, until a kernel is asked for by name)
+    int march_seg = 0;                // rows of their segments
     int sms = 0;                      // multiprocessors of the device
     int tile_h = 0;                   // with cpt == 2: rows of the small-lattice tiles (0: not used),
     int tile_levels = 0;              // and the steps one of their launches takes at most
@@ -317,6 +319,7 @@ void choose_tiles(lbm_ctx* h) {
         h->tile_levels = 4;
     }
 }
+int march_steps(const lbm_ctx* h);
 bool tiled(const lbm_ctx* h) { return h->tile_h > 0 && h->cpt == 2; }
 // Steps of the next launch of `left` >= 2: equal parts of at most tile_levels.
 int tile_steps(const lbm_ctx* h, int left) {
@@ -335,6 +338,16 @@ cudaError_t launch_tile(lbm_ctx* h, const void* src, void* dst, int levels, cuda
                                                    : lbm::launch_tile_bf16;
     return launch(src, dst, h->geo, h->k2, tx, ty, h->variant, h->bc, kTileRegion, h->tile_h,
                   levels, st, p, ls);
+}
+
+// The marching kernels' segments for the handle's layer and variant.
+void cut_march(lbm_ctx* h) {
+    if (!h->march) return;
+    const int nl = march_steps(h);
+    lbm::MarchGrid m = lbm::march_rectangle(h->geo, h->k2, h->variant, nl);
+    h->march_seg = lbm::march_segment(nl, h->sms, [&](int seg) {
+        return static_cast<long long>(lbm::march_cut(m, h->ny, seg));
+    });
 }
 
 // Set the handle's tile kernel up for its variant; without it, no tiles.
@@ -360,13 +373,13 @@ cudaError_t launch_march(lbm_ctx* h, const void* src, void* dst, cudaStream_t st
     switch (h->storage) {
         case LBM_F32:
             return (periodic ? lbm::launch_march_f32_periodic : lbm::launch_march_f32_dirichlet)(
-                src, dst, h->geo, h->k2, tx, ty, h->variant, h->sms, st, p);
+                src, dst, h->geo, h->k2, tx, ty, h->variant, h->march_seg, st, p);
         case LBM_F16DEV:
             return (periodic ? lbm::launch_march_f16_periodic : lbm::launch_march_f16_dirichlet)(
-                src, dst, h->geo, h->k2, tx, ty, h->variant, each, h->sms, st, p);
+                src, dst, h->geo, h->k2, tx, ty, h->variant, each, h->march_seg, st, p);
         case LBM_BF16DEV:
             return (periodic ? lbm::launch_march_bf16_periodic : lbm::launch_march_bf16_dirichlet)(
-                src, dst, h->geo, h->k2, tx, ty, h->variant, each, h->sms, st, p);
+                src, dst, h->geo, h->k2, tx, ty, h->variant, each, h->march_seg, st, p);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -619,6 +632,7 @@ int lbm_create(int nx, int ny, lbm_storage storage, double rho0, double ux0, dou
     h->march = h->cpt == 2 && !std::getenv("LBM_SPL") && !tma_env && march_pays(h, l2) &&
                cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device) ==
                    cudaSuccess;
+    cut_march(h);
     if (h->cpt == 2 && h->spl == 1 && !std::getenv("LBM_SPL") && !tma_env) choose_tiles(h);
     prepare_tiles(h);
     h->err.clear();
@@ -697,6 +711,7 @@ int lbm_set_sponge(lbm_handle h, lbm_variant variant, const double* chi_x, const
     lbm::zero_run(chi_x, h->nx, h->bulk[0], h->bulk[1]);
     lbm::zero_run(chi_y, h->ny, h->bulk[2], h->bulk[3]);
     refresh_consts(h);
+    cut_march(h);
     prepare_tiles(h);
     const double s_nu = h->rates.s[7];
     if ((variant == LBM_SPONGE_II || variant == LBM_SPONGE_III) && chi_max > 4.0 / s_nu)

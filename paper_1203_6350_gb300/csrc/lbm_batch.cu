@@ -29,6 +29,7 @@
 
 #include "lbm.h"
 #include "lbm_host.h"
+#include "lbm_march_cut.h"
 #include "lbm_step_tma.cuh"
 
 namespace lbm {
@@ -725,6 +726,17 @@ struct lbm_batch_ctx {
     std::vector<unsigned char> h_descs;
     std::vector<BatchTile> h_tiles;
     int h_ntiles[1 + 2 * lbm::kClasses] = {};  // host image of d_ntiles (256 bytes allocated)
+    // Marching launches of large two-step batches: what a launch does not change of the
+    // instances, grouped by variant and at most kMarchItems to a launch
+    struct MarchGroup {
+        int variant;
+        std::vector<int> ids;
+        std::vector<lbm::MarchItem> items;
+    };
+    bool march = false;
+    int sms = 0;
+    std::vector<MarchGroup> march_groups;
+    lbm::MarchBatch march_params;  // the launch being built
     int class_mask = 0;  // classes with tiles
     int graph_mask = 0;  // classes the captured graph launches
     // TMA staging of the two-step input (FP32 batches, Dirichlet instances)
@@ -932,6 +944,104 @@ cudaError_t compute_grid(lbm_batch_ctx* b) {
     return cudaSuccess;
 }
 
+// Steps of one marching launch.
+int march_levels(const lbm_batch_ctx* b) { return b->storage == LBM_F32 ? 3 : 2; }
+
+// Whether marching launches are the faster ones for this batch (Dirichlet instances,
+// two steps per launch chosen, no environment variable that names the tile kernels'
+// loads).  Measured against the tile kernels, ratio of throughputs by count and sides:
+// FP32 256 of 64-1024 1.32, 64 of 64-1024 1.42, 32 of 64-512 1.28, 8 of 256-1024 1.52, 8 of
+// 200-300 1.13, but 32 of 64-256 0.91 and 64 of 64-128 0.91; FP16 1.14, 1.34, 1.33, 1.62,
+// 1.39, 1.29 and 1.04, 128 of 64-128 0.71.  Small instances leave a warp little but edges
+// and constants that change with every block: the line is drawn at their mean size.
+bool march_pays(const lbm_batch_ctx* b) {
+    if (b->storage == LBM_F64 || b->cpt != 2 || b->spl != 2 || std::getenv("LBM_BATCH_TMA"))
+        return false;
+    long long cells = 0, count = 0;
+    for (const auto& kv : b->insts) {
+        const Instance& in = kv.second;
+        if (in.bc != LBM_BC_DIRICHLET_EQ) return false;
+        if (!in.initialised) continue;
+        cells += static_cast<long long>(in.nx) * in.ny;
+        ++count;
+    }
+    return count > 0 && cells >= count * (b->storage == LBM_F32 ? 36000 : 16000);
+}
+
+// Group the initialised instances for marching launches.
+void build_march_groups(lbm_batch_ctx* b) {
+    b->march_groups.clear();
+    b->march = march_pays(b);
+    if (!b->march) return;
+    const int nl = march_levels(b);
+    std::map<int, std::vector<int>> by_variant;
+    for (const auto& kv : b->insts)
+        if (kv.second.initialised) by_variant[kv.second.variant].push_back(kv.first);
+    for (const auto& [variant, ids] : by_variant) {
+        const size_t groups = (ids.size() + lbm::kMarchItems - 1) / lbm::kMarchItems;
+        for (size_t q = 0; q < groups; ++q) {
+            lbm_batch_ctx::MarchGroup g;
+            g.variant = variant;
+            for (size_t i = q; i < ids.size(); i += groups) g.ids.push_back(ids[i]);
+            for (const int id : g.ids) {
+                const Instance& in = b->insts.at(id);
+                lbm::MarchItem it{};
+                it.k = consts_of<lbm::F2>(in);
+                it.tx = static_cast<const AxisCoef<float>*>(in.tabs);
+                it.ty = it.tx + in.nx;
+                it.nx = in.nx;
+                it.ny = in.ny;
+                it.pitch = static_cast<int>(in.geo.pitch);
+                it.plane = static_cast<unsigned>(in.geo.plane);
+                it.grid = lbm::march_rectangle(in.geo, it.k, in.variant, nl);
+                g.items.push_back(it);
+            }
+            lbm::march_segment(nl, b->sms, [&](int seg) {
+                long long blocks = 0;
+                for (auto& it : g.items) blocks += lbm::march_cut(it.grid, it.ny, seg);
+                return blocks;
+            });
+            b->march_groups.push_back(std::move(g));
+        }
+    }
+}
+
+// Advance every active instance by the d steps of a marching launch from global step s0;
+// *done = false (and nothing launched) when one of them ends within it.
+cudaError_t launch_march(lbm_batch_ctx* b, int64_t s0, int d, int pdl, bool* done) {
+    *done = true;
+    for (const auto& kv : b->insts) {
+        const Instance& in = kv.second;
+        const int64_t end = in.start + in.budget;
+        if (in.initialised && s0 >= in.start && s0 < end && end - s0 < d) *done = false;
+    }
+    if (!*done) return cudaSuccess;
+    const auto launch = b->storage == LBM_F32      ? lbm::launch_march_batch_f32
+                        : b->storage == LBM_F16DEV ? lbm::launch_march_batch_f16
+                                                   : lbm::launch_march_batch_bf16;
+    cudaError_t e = cudaSuccess;
+    for (const auto& g : b->march_groups) {
+        lbm::MarchBatch& p = b->march_params;
+        p.count = p.blocks = 0;
+        p.sms = b->sms;
+        for (size_t i = 0; i < g.ids.size(); ++i) {
+            const Instance& in = b->insts.at(g.ids[i]);
+            if (s0 < in.start || s0 >= in.start + in.budget) continue;
+            lbm::MarchItem& it = p.item[p.count++];
+            it = g.items[i];
+            it.src = in.buf[in.launched & 1];
+            it.dst = in.buf[1 - (in.launched & 1)];
+            it.block0 = p.blocks;
+            p.blocks += it.grid.blocks;
+        }
+        if (p.count == 0) continue;
+        e = launch(p, g.variant, b->stream, pdl);
+        if (e != cudaSuccess) return e;
+        pdl = 1;
+    }
+    return e;
+}
+
 // Rebuild the descriptor array and the tile table on the device (stream-ordered).
 int sync_tables(lbm_batch_ctx* b) {
     if (!b->dirty) return LBM_OK;
@@ -965,6 +1075,7 @@ int sync_tables(lbm_batch_ctx* b) {
         for (int y0 = 0; y0 < in.ny; y0 += ty)
             for (int x0 = 0; x0 < in.nx; x0 += tx) out.push_back(BatchTile{di, x0, y0, 0});
     }
+    build_march_groups(b);
     // tensor maps of both buffers of every Dirichlet instance (FP32 two-step batches)
     if (b->tma && b->spl == 2) {
         b->h_maps.assign(2 * b->dense.size(), CUtensorMap{});
@@ -1122,6 +1233,7 @@ int lbm_batch_create(lbm_storage storage, void* cuda_stream, const lbm_allocator
         b->custom_alloc = true;
     }
     cudaError_t e = cudaGetDevice(&b->device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, b->device);
     if (e == cudaSuccess) e = compute_grid(b);
     if (e != cudaSuccess) {
         delete b;
@@ -1383,6 +1495,29 @@ int lbm_batch_step(lbm_batch b, int nsteps) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     e = cudaStreamIsCapturing(b->stream, &cs);
     if (e != cudaSuccess) return bfail(b, LBM_ERR_CUDA, "cudaStreamIsCapturing");
+    // Marching launches carry the instances' buffers, as the host knows them, in their
+    // parameters; a captured stream is replayed with others, so it keeps to the kernels that
+    // read them on the device.
+    int step_off = 0, launch_off = 0;
+    for (bool march = b->march && cs == cudaStreamCaptureStatusNone;
+         march && nsteps >= march_levels(b);) {
+        const int d = march_levels(b);
+        e = launch_march(b, b->step + step_off, d, launch_off > 0, &march);
+        if (e != cudaSuccess) return bfail(b, LBM_ERR_CUDA, std::string("batch launch: ") + cudaGetErrorString(e));
+        if (!march) break;
+        account(b, b->step + step_off, d, 1);
+        step_off += d;
+        ++launch_off;
+        nsteps -= d;
+    }
+    if (launch_off > 0) {
+        lbm::advance_counters_kernel<<<1, 1, 0, b->stream>>>(b->d_counters, step_off, launch_off);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return bfail(b, LBM_ERR_CUDA, std::string("batch advance: ") + cudaGetErrorString(e));
+        b->step += step_off;
+        b->launches += launch_off;
+        step_off = launch_off = 0;
+    }
     if (cs == cudaStreamCaptureStatusNone && nsteps >= kBatchChunk) {
         e = ensure_batch_graph(b);
         if (e != cudaSuccess) return bfail(b, LBM_ERR_CUDA, std::string("batch graph: ") + cudaGetErrorString(e));
@@ -1396,7 +1531,6 @@ int lbm_batch_step(lbm_batch b, int nsteps) {
             nsteps -= kBatchChunk;
         }
     }
-    int step_off = 0, launch_off = 0;
     while (nsteps > 0) {
         const int d = (b->spl == 2 && nsteps >= 2) ? 2 : 1;
         e = launch_batch(b, b->stream, d, step_off, launch_off, launch_off > 0);

@@ -268,31 +268,31 @@ cudaError_t launch_step_tb2_bf16(const void* src, void* dst, const Geometry& g,
                                  int pdl);
 
 // Several steps per launch by marching warps (lbm_march.cuh): src holds time t,
-// dst receives t + 3 (FP32, and 16-bit storage with each_level) or t + 2.  sms:
-// multiprocessors of the device.
+// dst receives t + 3 (FP32, and 16-bit storage with each_level) or t + 2.  seg: rows of
+// a segment (march_segment).
 cudaError_t launch_march_f32_dirichlet(const void* src, void* dst, const Geometry& g,
                                    const StepConst<F2>& k, const AxisCoef<float>* tx,
-                                   const AxisCoef<float>* ty, int variant, int sms,
+                                   const AxisCoef<float>* ty, int variant, int seg,
                                    cudaStream_t st, int pdl);
 cudaError_t launch_march_f32_periodic(const void* src, void* dst, const Geometry& g,
                                    const StepConst<F2>& k, const AxisCoef<float>* tx,
-                                   const AxisCoef<float>* ty, int variant, int sms,
+                                   const AxisCoef<float>* ty, int variant, int seg,
                                    cudaStream_t st, int pdl);
 cudaError_t launch_march_f16_dirichlet(const void* src, void* dst, const Geometry& g,
                                    const StepConst<F2>& k, const AxisCoef<float>* tx,
-                                   const AxisCoef<float>* ty, int variant, bool each_level, int sms,
+                                   const AxisCoef<float>* ty, int variant, bool each_level, int seg,
                                    cudaStream_t st, int pdl);
 cudaError_t launch_march_f16_periodic(const void* src, void* dst, const Geometry& g,
                                    const StepConst<F2>& k, const AxisCoef<float>* tx,
-                                   const AxisCoef<float>* ty, int variant, bool each_level, int sms,
+                                   const AxisCoef<float>* ty, int variant, bool each_level, int seg,
                                    cudaStream_t st, int pdl);
 cudaError_t launch_march_bf16_dirichlet(const void* src, void* dst, const Geometry& g,
                                    const StepConst<F2>& k, const AxisCoef<float>* tx,
-                                   const AxisCoef<float>* ty, int variant, bool each_level, int sms,
+                                   const AxisCoef<float>* ty, int variant, bool each_level, int seg,
                                    cudaStream_t st, int pdl);
 cudaError_t launch_march_bf16_periodic(const void* src, void* dst, const Geometry& g,
                                    const StepConst<F2>& k, const AxisCoef<float>* tx,
-                                   const AxisCoef<float>* ty, int variant, bool each_level, int sms,
+                                   const AxisCoef<float>* ty, int variant, bool each_level, int seg,
                                    cudaStream_t st, int pdl);
 
 // Several steps (levels >= 2) per launch on tiles of h rows in regions of rw = 32 or 64

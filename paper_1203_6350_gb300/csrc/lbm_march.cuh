@@ -39,32 +39,10 @@
 // 4096^2: 183 before, 238 with it.
 #pragma once
 
+#include "lbm_march_cut.h"
 #include "lbm_step2.cuh"
 
 namespace lbm {
-
-// Columns computed twice at each end of a strip of NL levels (NL - 1, kept even).
-__host__ __device__ constexpr int march_halo(int nl) { return nl / 2 * 2; }
-// Columns a strip stores.
-__host__ __device__ constexpr int march_width(int nl) { return 64 - 2 * march_halo(nl); }
-// Resident warps per SM: two levels fit 128 registers, three fit 168 (at 128 they
-// spill: 188 in place of 242 GLUPS at 4096^2 FP32).
-__host__ __device__ constexpr int march_per_sm(int nl) { return nl == 2 ? 16 : 12; }
-constexpr int kMarchChunks = 17;              // chunks of four elements per staged plane-row
-constexpr int kMarchStage = 9 * kMarchChunks; // chunks per ring slot
-constexpr int kMarchRow = 4 * kMarchChunks;   // elements per staged plane-row
-constexpr int kMarchSlots = 3;                // ring slots: two rows ahead of the walk
-constexpr int kMarchMaxSeg = 64;              // rows of a segment at most
-
-// How a launch is cut (march_grid): columns [s0, s1) of strips and rows
-// [y0, y1) are the rectangle without checks.
-struct MarchGrid {
-    int strips, s0, s1, y0, y1;
-    int seg, seg_gen;      // rows per segment, in the rectangle and outside it
-    int n_side, n_middle;  // blocks of the side strips, and of the rows above and below
-    int n_top;             // segments above the rectangle
-    int blocks;
-};
 
 // What the next level needs of the rows that one level has produced.
 struct MarchLine {
@@ -343,86 +321,57 @@ __device__ __forceinline__ void march(const T* __restrict__ src, T* __restrict__
     }
 }
 
+// Block b of a launch: its strip, its rows, and whether it lies in the rectangle.
+struct MarchWalk {
+    int strip, ya, yb;
+    bool fast;
+};
+__device__ __forceinline__ MarchWalk march_walk(const MarchGrid& g, int b, int ny) {
+    const int nm = g.s1 - g.s0;
+    MarchWalk w;
+    if (b >= g.n_side + g.n_middle) {
+        b -= g.n_side + g.n_middle;
+        w.strip = g.s0 + b % nm;
+        w.ya = g.y0 + b / nm * g.seg;
+        w.yb = min(w.ya + g.seg, g.y1);
+        w.fast = true;
+        return w;
+    }
+    int end = ny;
+    if (b < g.n_side) {
+        const int ns = g.s0 + g.strips - g.s1;
+        w.strip = b % ns;
+        if (w.strip >= g.s0) w.strip += nm;
+        w.ya = b / ns * g.seg_gen;
+    } else {
+        b -= g.n_side;
+        const int q = b / nm;
+        w.strip = g.s0 + b % nm;
+        w.ya = q < g.n_top ? q * g.seg_gen : g.y1 + (q - g.n_top) * g.seg_gen;
+        if (q < g.n_top) end = g.y0;
+    }
+    w.yb = min(w.ya + g.seg_gen, end);
+    w.fast = false;
+    return w;
+}
+
 template <typename T, int VAR, int BC, int NL, bool RND>
 __global__ void __launch_bounds__(32, march_per_sm(NL))
     march_kernel(const T* __restrict__ src, T* __restrict__ dst, int nx, int ny, int pitch,
                  unsigned plane, StepConst<F2> k, const AxisCoef<float>* __restrict__ tx,
                  const AxisCoef<float>* __restrict__ ty, MarchGrid g) {
-    constexpr int kMarchW = march_width(NL);
     __shared__ __align__(16) T ring[kMarchSlots * 4 * kMarchStage];
     __shared__ float4 rows_y[VAR == kNone ? 1 : kMarchMaxSeg + 2 * (NL - 1)];
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const size_t plane_bytes = static_cast<size_t>(plane) * sizeof(T);
-    int b = blockIdx.x;
-    if (b >= g.n_side + g.n_middle) {
-        b -= g.n_side + g.n_middle;
-        const int nm = g.s1 - g.s0, ya = g.y0 + b / nm * g.seg;
+    const MarchWalk w = march_walk(g, blockIdx.x, ny);
+    if (w.fast)
         march<T, VAR, BC, NL, RND, true>(src, dst, nx, ny, pitch, plane_bytes, k, tx, ty,
-                                         (g.s0 + b % nm) * kMarchW, ya, min(ya + g.seg, g.y1),
-                                         ring, rows_y);
-    } else {
-        int s, ya, end = ny;
-        if (b < g.n_side) {
-            const int ns = g.s0 + g.strips - g.s1;
-            s = b % ns;
-            if (s >= g.s0) s += g.s1 - g.s0;
-            ya = b / ns * g.seg_gen;
-        } else {
-            b -= g.n_side;
-            const int nm = g.s1 - g.s0, q = b / nm;
-            s = g.s0 + b % nm;
-            ya = q < g.n_top ? q * g.seg_gen : g.y1 + (q - g.n_top) * g.seg_gen;
-            if (q < g.n_top) end = g.y0;
-        }
+                                         w.strip * march_width(NL), w.ya, w.yb, ring, rows_y);
+    else
         march<T, VAR, BC, NL, RND, false>(src, dst, nx, ny, pitch, plane_bytes, k, tx, ty,
-                                          s * kMarchW, ya, min(ya + g.seg_gen, end), ring, rows_y);
-    }
+                                          w.strip * march_width(NL), w.ya, w.yb, ring, rows_y);
     asm volatile("griddepcontrol.launch_dependents;");
-}
-
-// Cut the lattice into strips and segments for a launch of NL levels.
-inline MarchGrid march_grid(const Geometry& g, const StepConst<F2>& k, int variant, int nl,
-                            int sms) {
-    MarchGrid m{};
-    const int kMarchW = march_width(nl), kMarchHalo = march_halo(nl);
-    m.strips = (g.nx + kMarchW - 1) / kMarchW;
-    // strips whose staged columns lie in the lattice and whose cells lie in the bulk
-    const bool layer = variant != kNone;
-    auto fast = [&](int s) {
-        const int x = s * kMarchW;
-        return x - 4 >= 0 && x - 4 + kMarchRow <= g.nx &&
-               (!layer || (x - kMarchHalo >= k.bulk_x0 && x - kMarchHalo + 64 <= k.bulk_x1));
-    };
-    m.s0 = 0;
-    while (m.s0 < m.strips && !fast(m.s0)) ++m.s0;
-    m.s1 = m.s0;
-    while (m.s1 < m.strips && fast(m.s1)) ++m.s1;
-    // rows whose segments pull rows of the lattice and collide rows of the bulk
-    m.y0 = layer && k.bulk_y0 - 1 > 0 ? k.bulk_y0 - 1 + nl : nl;
-    m.y1 = (layer && k.bulk_y1 + 1 < g.ny ? k.bulk_y1 + 1 : g.ny) - nl;
-    if (m.y1 <= m.y0 || m.s1 == m.s0) {
-        m.s0 = m.s1 = m.strips;
-        m.y0 = m.y1 = g.ny;
-    }
-    const long long slots = static_cast<long long>(sms) * march_per_sm(nl);
-    const auto blocks = [&](int seg, int seg_gen) {
-        const long long ns = m.s0 + m.strips - m.s1, nm = m.s1 - m.s0;
-        const auto segs = [](int n, int s) { return (n + s - 1) / s; };
-        m.seg = seg;
-        m.seg_gen = seg_gen;
-        m.n_side = static_cast<int>(ns * segs(g.ny, seg_gen));
-        m.n_top = nm ? segs(m.y0, seg_gen) : 0;
-        m.n_middle = nm ? static_cast<int>(nm * (m.n_top + segs(g.ny - m.y1, seg_gen))) : 0;
-        m.blocks = static_cast<int>(m.n_side + m.n_middle + nm * segs(m.y1 - m.y0, seg));
-        return m.blocks;
-    };
-    // The shortest segments whose blocks fit the device's slots k times, for the
-    // smallest k that keeps them within kMarchMaxSeg rows: the last wave is then
-    // nearly full, and few rows are computed twice.  Outside the rectangle a row
-    // costs about 1.5 times as much, so segments are 5/8 as long there.
-    for (long long waves = 1;; ++waves)
-        for (int seg = 4; seg <= kMarchMaxSeg; ++seg)
-            if (blocks(seg, seg * 5 / 8) <= waves * slots) return m;
 }
 
 // Advance NL steps: src holds time t, dst receives t + NL; pdl as for the one-step
@@ -430,9 +379,10 @@ inline MarchGrid march_grid(const Geometry& g, const StepConst<F2>& k, int varia
 template <typename T, int BC, int NL, bool RND>
 cudaError_t launch_march_t(const void* src, void* dst, const Geometry& g, const StepConst<F2>& k,
                            const AxisCoef<float>* tx, const AxisCoef<float>* ty, int variant,
-                           int sms, cudaStream_t st, int pdl) {
+                           int seg, cudaStream_t st, int pdl) {
     if (9 * g.plane >= (1ll << 32)) return cudaErrorInvalidValue;
-    const MarchGrid m = march_grid(g, k, variant, NL, sms);
+    MarchGrid m = march_rectangle(g, k, variant, NL);
+    march_cut(m, g.ny, seg);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(m.blocks);
     cfg.blockDim = dim3(32);

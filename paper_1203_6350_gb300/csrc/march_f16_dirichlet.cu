@@ -8,10 +8,10 @@ namespace lbm {
 cudaError_t launch_march_f16_dirichlet(const void* src, void* dst, const Geometry& g,
                                    const StepConst<F2>& k, const AxisCoef<float>* tx,
                                    const AxisCoef<float>* ty, int variant, bool each_level,
-                                   int sms, cudaStream_t st, int pdl) {
+                                   int seg, cudaStream_t st, int pdl) {
     if (each_level)
-        return launch_march_t<__half, kDirichlet, 3, true>(src, dst, g, k, tx, ty, variant, sms, st, pdl);
-    return launch_march_t<__half, kDirichlet, 2, false>(src, dst, g, k, tx, ty, variant, sms, st, pdl);
+        return launch_march_t<__half, kDirichlet, 3, true>(src, dst, g, k, tx, ty, variant, seg, st, pdl);
+    return launch_march_t<__half, kDirichlet, 2, false>(src, dst, g, k, tx, ty, variant, seg, st, pdl);
 }
 
 }  // namespace lbm
