@@ -161,6 +161,24 @@ __device__ __forceinline__ float rcp_eq(float x) {
 __device__ __forceinline__ double rcp_eq(double x) { return __drcp_rn(x); }
 __device__ __forceinline__ F2 rcp_eq(F2 x) { return f2(rcp_eq(f2_lo(x)), rcp_eq(f2_hi(x))); }
 
+// 2 a - b and b - 2 a.  The doubling is exact, so one fused instruction rounds as the
+// two do.  FP64 only, whose step is bound by its FP64 instructions: the FP32 forms stay
+// as they are, since the code generator's other choices hang on them.
+template <typename V>
+__device__ __forceinline__ V twice_minus(V a, V b) {
+    if constexpr (std::is_same<V, double>::value)
+        return __fma_rn(2.0, a, -b);
+    else
+        return (a + a) - b;
+}
+template <typename V>
+__device__ __forceinline__ V minus_twice(V b, V a) {
+    if constexpr (std::is_same<V, double>::value)
+        return __fma_rn(-2.0, a, b);
+    else
+        return b - (a + a);
+}
+
 // Moments m = M g (App. A.1), written as sums and differences.
 template <typename V>
 __device__ __forceinline__ void moments9(const V (&g)[9], V (&m)[9]) {
@@ -173,8 +191,8 @@ __device__ __forceinline__ void moments9(const V (&g)[9], V (&m)[9]) {
     m[0] = g[0] + s14 + s58;                                 // rho'
     m[1] = a13 + bpc;                                        // j_x'
     m[2] = a24 + bmc;                                        // j_y'
-    m[3] = (s58 + s58) - fmadd(lit<V>(4.0f), g[0], s14);     // e: 2 s58 - s14 - 4 g0
-    m[4] = fmadd(lit<V>(4.0f), g[0], s58) - (s14 + s14);     // epsilon: 4 g0 - 2 s14 + s58
+    m[3] = twice_minus(s58, fmadd(lit<V>(4.0f), g[0], s14));  // e: 2 s58 - s14 - 4 g0
+    m[4] = minus_twice(fmadd(lit<V>(4.0f), g[0], s58), s14);  // epsilon: 4 g0 - 2 s14 + s58
     m[5] = fmadd(lit<V>(-2.0f), a13, bpc);                   // q_x
     m[6] = fmadd(lit<V>(-2.0f), a24, bmc);                   // q_y
     m[7] = p13 - p24;                                        // p_xx
@@ -235,6 +253,10 @@ __device__ __forceinline__ V scale_conserved(V v, const StepConst<V>& k, int row
 template <typename T>
 struct UnbiasedScale {
     static constexpr bool value = true;
+};
+template <>  // (its residual is zero, and three FP64 products fewer are 3 % of the step)
+struct UnbiasedScale<double> {
+    static constexpr bool value = false;
 };
 template <>
 struct UnbiasedScale<__half> {
