@@ -28,6 +28,7 @@
 
 #include "lbm.h"
 #include "lbm_host.h"
+#include "lbm_read.cuh"
 
 namespace {
 
@@ -283,47 +284,60 @@ __global__ void __launch_bounds__(kBX * kBY)
     for (int i = 0; i < kQ; ++i) dst[plane_off<NARROW>(i, g.plane, o)] = f[i];
 }
 
-// Slot x of plane i <- f^eq_i(rho, u at x + c_i) - f^eq_i(rho0, u0) (the
-// wrapped cell when periodic; 0 when x + c_i is outside, a slot no pull reads).
-// Fields are FP64 [nz][ny][nx] on the device.
-template <typename T>
-__global__ void d3_init_kernel(T* __restrict__ dst, D3Geom g, double rho0, double ux0,
-                               double uy0, double uz0, int bc, const double* __restrict__ rho,
-                               const double* __restrict__ ux, const double* __restrict__ uy,
-                               const double* __restrict__ uz) {
+// Store population i of cell (x, y, z) in the slot its first pull reads, and zero in the
+// cell's own slot where that one's source lies outside the lattice.  Every slot is
+// written once.
+template <typename T, int BC>
+__device__ __forceinline__ void d3_put(T* __restrict__ dst, const D3Geom& g, int i, int x, int y,
+                                       int z, double v) {
+    const int cx = d3cx(i), cy = d3cy(i), cz = d3cz(i);
+    int tx = x - cx, ty = y - cy, tz = z - cz;  // the slot that cell (x, y, z) pulls
+    T* plane = dst + static_cast<size_t>(i) * g.plane;
+    if (BC == LBM_BC_PERIODIC) {
+        tx = wrap(tx, g.nx);
+        ty = wrap(ty, g.ny);
+        tz = wrap(tz, g.nz);
+    } else {
+        const int sx = x + cx, sy = y + cy, sz = z + cz;
+        if (sx < 0 || sx >= g.nx || sy < 0 || sy >= g.ny || sz < 0 || sz >= g.nz)
+            plane[(static_cast<unsigned>(z) * g.ny + y) * g.pitch + x] = T(0);
+        if (tx < 0 || tx >= g.nx || ty < 0 || ty >= g.ny || tz < 0 || tz >= g.nz) return;
+    }
+    plane[(static_cast<unsigned>(tz) * g.ny + ty) * g.pitch + tx] = static_cast<T>(v);
+}
+
+// f^eq_i(rho, u) - f^eq_i(rho0, u0) of every cell (fields FP64 [nz][ny][nx] on the device).
+// Bound by FP64 instructions, so a cell is computed once, what its populations share
+// among it, and not each population from its source cell.  lbm3_init_equilibrium of 128^3
+// FP32 from host fields: 2.09 ms with that and an allocation per call, 1.30 ms now.
+template <typename T, int BC>
+__global__ void __launch_bounds__(128)
+    d3_init_kernel(T* __restrict__ dst, D3Geom g, double rho0, double ux0, double uy0, double uz0,
+                   const double* __restrict__ rho, const double* __restrict__ ux,
+                   const double* __restrict__ uy, const double* __restrict__ uz) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y;
     const int z = blockIdx.z;
     if (x >= g.nx) return;
+    const size_t c = (static_cast<size_t>(z) * g.ny + y) * g.nx + x;
+    const double r = rho[c], u[3] = {ux[c], uy[c], uz[c]}, u0[3] = {ux0, uy0, uz0};
     const double w[3] = {2.0 / 9.0, 1.0 / 9.0, 1.0 / 72.0};
-    const double u0[3] = {ux0, uy0, uz0};
-    const unsigned o = (static_cast<unsigned>(z) * g.ny + y) * g.pitch + x;
+#pragma unroll
     for (int i = 0; i < kQ; ++i) {
-        int sx = x + d3cx(i), sy = y + d3cy(i), sz = z + d3cz(i);
-        double v = 0.0;
-        if (bc == LBM_BC_PERIODIC) {
-            sx = wrap(sx, g.nx);
-            sy = wrap(sy, g.ny);
-            sz = wrap(sz, g.nz);
+        const int ci[3] = {d3cx(i), d3cy(i), d3cz(i)};
+        // f^eq(rho, u) - f^eq(rho0, u0) over w_i, term by term
+        double cu = 0, cu0 = 0, uu = 0, uu0 = 0;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            cu += ci[a] * u[a];
+            cu0 += ci[a] * u0[a];
+            uu += u[a] * u[a];
+            uu0 += u0[a] * u0[a];
         }
-        if (sx >= 0 && sx < g.nx && sy >= 0 && sy < g.ny && sz >= 0 && sz < g.nz) {
-            const size_t c = (static_cast<size_t>(sz) * g.ny + sy) * g.nx + sx;
-            const double r = rho[c], u[3] = {ux[c], uy[c], uz[c]};
-            const int ci[3] = {d3cx(i), d3cy(i), d3cz(i)};
-            // f^eq(rho, u) - f^eq(rho0, u0) over w_i, term by term
-            double cu = 0, cu0 = 0, uu = 0, uu0 = 0;
-            for (int a = 0; a < 3; ++a) {
-                cu += ci[a] * u[a];
-                cu0 += ci[a] * u0[a];
-                uu += u[a] * u[a];
-                uu0 += u0[a] * u0[a];
-            }
-            const double dr = r - rho0;
-            const double dlin = dr + 3.0 * (r * cu - rho0 * cu0);
-            const double dquad = 4.5 * (r * cu * cu - rho0 * cu0 * cu0) - 1.5 * (r * uu - rho0 * uu0);
-            v = w[i == 0 ? 0 : (i < 7 ? 1 : 2)] * (dlin + dquad);
-        }
-        dst[static_cast<size_t>(i) * g.plane + o] = static_cast<T>(v);
+        const double dr = r - rho0;
+        const double dlin = dr + 3.0 * (r * cu - rho0 * cu0);
+        const double dquad = 4.5 * (r * cu * cu - rho0 * cu0 * cu0) - 1.5 * (r * uu - rho0 * uu0);
+        d3_put<T, BC>(dst, g, i, x, y, z, w[i == 0 ? 0 : (i < 7 ? 1 : 2)] * (dlin + dquad));
     }
 }
 
@@ -332,6 +346,7 @@ template <typename T>
 __device__ __forceinline__ void d3_pulled_moments(const T* __restrict__ src, const D3Geom& g,
                                                   int bc, int x, int y, int z, double (&m)[4]) {
     m[0] = m[1] = m[2] = m[3] = 0.0;
+#pragma unroll
     for (int i = 0; i < kQ; ++i) {
         int sx = x - d3cx(i), sy = y - d3cy(i), sz = z - d3cz(i);
         double v = 0.0;
@@ -341,12 +356,12 @@ __device__ __forceinline__ void d3_pulled_moments(const T* __restrict__ src, con
             sz = wrap(sz, g.nz);
         }
         if (sx >= 0 && sx < g.nx && sy >= 0 && sy < g.ny && sz >= 0 && sz < g.nz)
-            v = static_cast<double>(src[static_cast<size_t>(i) * g.plane +
-                                        (static_cast<unsigned>(sz) * g.ny + sy) * g.pitch + sx]);
+            v = lbm::widen(src[static_cast<size_t>(i) * g.plane +
+                               (static_cast<unsigned>(sz) * g.ny + sy) * g.pitch + sx]);
         m[0] += v;
-        m[1] += d3cx(i) * v;
-        m[2] += d3cy(i) * v;
-        m[3] += d3cz(i) * v;
+        if (d3cx(i) != 0) m[1] += d3cx(i) * v;
+        if (d3cy(i) != 0) m[2] += d3cy(i) * v;
+        if (d3cz(i) != 0) m[3] += d3cz(i) * v;
     }
 }
 
@@ -366,9 +381,10 @@ __global__ void d3_moments_kernel(const T* __restrict__ src, D3Geom g, double rh
     const double r = rho0 + m[0];
     const size_t c = (static_cast<size_t>(z) * g.ny + y) * g.nx + x;
     rho[c] = m[0];
-    ux[c] = (rho0 * ux0 + m[1]) / r;
-    uy[c] = (rho0 * uy0 + m[2]) / r;
-    uz[c] = (rho0 * uz0 + m[3]) / r;
+    const lbm::Reciprocal inv = lbm::reciprocal(r, static_cast<float>(r));
+    ux[c] = lbm::quotient(rho0 * ux0 + m[1], inv, isfinite(m[1]));
+    uy[c] = lbm::quotient(rho0 * uy0 + m[2], inv, isfinite(m[2]));
+    uz[c] = lbm::quotient(rho0 * uz0 + m[3], inv, isfinite(m[3]));
 }
 
 constexpr int kD3Diag = 7;           // sums of lbm3_diagnostics
@@ -471,6 +487,34 @@ struct lbm3_ctx {
 namespace {
 
 thread_local std::string g_lbm3_error;
+
+// Device room for four FP64 fields on the handle's stream.  The population buffer that
+// holds no state has 60 or 120 bytes per cell and is overwritten by the next step,
+// so it serves where its rows have no padding (which stays as it is); otherwise an
+// allocation for the call.
+struct FieldScratch {
+    double* d = nullptr;
+    bool owned = false;
+    cudaStream_t stream;
+    explicit FieldScratch(lbm3_ctx* h) : stream(h->stream) {
+        if (h->g.pitch == h->nx) {
+            d = static_cast<double*>(h->buf[h->cur ^ 1]);
+            return;
+        }
+        const size_t cells = static_cast<size_t>(h->nx) * h->ny * h->nz;
+        if (cudaMallocAsync(&d, 4 * cells * sizeof(double), stream) == cudaSuccess) {
+            owned = true;
+        } else {
+            cudaGetLastError();
+            d = nullptr;
+        }
+    }
+    void release() {
+        if (owned) cudaFreeAsync(d, stream);
+        owned = false;
+    }
+    ~FieldScratch() { release(); }
+};
 
 int fail3(lbm3_ctx* h, int code, const std::string& msg) {
     if (h) h->err = msg;
@@ -692,32 +736,34 @@ int lbm3_init_equilibrium(lbm3_handle h, const double* rho, const double* ux, co
     if (!h) return fail3(nullptr, LBM_ERR_ARG, "NULL handle");
     if (!rho || !ux || !uy || !uz) return fail3(h, LBM_ERR_ARG, "NULL field");
     const size_t cells = static_cast<size_t>(h->nx) * h->ny * h->nz;
-    double* d = nullptr;
-    if (cudaMallocAsync(&d, 4 * cells * sizeof(double), h->stream) != cudaSuccess) {
-        cudaGetLastError();
-        return fail3(h, LBM_ERR_OOM, "device allocation failed");
-    }
+    FieldScratch scratch(h);
+    double* d = scratch.d;
+    if (!d) return fail3(h, LBM_ERR_OOM, "device allocation failed");
     const double* src[4] = {rho, ux, uy, uz};
     cudaError_t e = cudaSuccess;
     for (int a = 0; a < 4 && e == cudaSuccess; ++a)
         e = cudaMemcpyAsync(d + a * cells, src[a], cells * sizeof(double), cudaMemcpyHostToDevice,
                             h->stream);
     if (e == cudaSuccess) {
-        const dim3 block(128), grid((h->nx + 127) / 128, h->ny, h->nz);
+        const auto launch = [&](auto kernel, auto* dst) {
+            const dim3 block(128), grid((h->nx + 127) / 128, h->ny, h->nz);
+            kernel<<<grid, block, 0, h->stream>>>(dst, h->g, h->rho0, h->u0[0], h->u0[1], h->u0[2],
+                                                  d, d + cells, d + 2 * cells, d + 3 * cells);
+        };
+        const bool periodic = h->bc == LBM_BC_PERIODIC;
         if (h->storage == LBM_F64)
-            d3_init_kernel<double><<<grid, block, 0, h->stream>>>(
-                static_cast<double*>(h->buf[0]), h->g, h->rho0, h->u0[0], h->u0[1], h->u0[2],
-                h->bc, d, d + cells, d + 2 * cells, d + 3 * cells);
+            launch(periodic ? d3_init_kernel<double, LBM_BC_PERIODIC>
+                            : d3_init_kernel<double, LBM_BC_DIRICHLET_EQ>,
+                   static_cast<double*>(h->buf[h->cur]));
         else
-            d3_init_kernel<float><<<grid, block, 0, h->stream>>>(
-                static_cast<float*>(h->buf[0]), h->g, h->rho0, h->u0[0], h->u0[1], h->u0[2],
-                h->bc, d, d + cells, d + 2 * cells, d + 3 * cells);
+            launch(periodic ? d3_init_kernel<float, LBM_BC_PERIODIC>
+                            : d3_init_kernel<float, LBM_BC_DIRICHLET_EQ>,
+                   static_cast<float*>(h->buf[h->cur]));
         e = cudaGetLastError();
     }
-    cudaFreeAsync(d, h->stream);
+    scratch.release();
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) return fail3(h, LBM_ERR_CUDA, cudaGetErrorString(e));
-    h->cur = 0;
     h->time = 0;
     h->ready = true;
     return LBM_OK;
@@ -742,11 +788,9 @@ int lbm3_moments(lbm3_handle h, double* rho_dev, double* ux, double* uy, double*
     if (!rho_dev || !ux || !uy || !uz) return fail3(h, LBM_ERR_ARG, "NULL output");
     if (!h->ready) return fail3(h, LBM_ERR_STATE, "moments before lbm3_init_equilibrium");
     const size_t cells = static_cast<size_t>(h->nx) * h->ny * h->nz;
-    double* d = nullptr;
-    if (cudaMallocAsync(&d, 4 * cells * sizeof(double), h->stream) != cudaSuccess) {
-        cudaGetLastError();
-        return fail3(h, LBM_ERR_OOM, "device allocation failed");
-    }
+    FieldScratch scratch(h);
+    double* d = scratch.d;
+    if (!d) return fail3(h, LBM_ERR_OOM, "device allocation failed");
     const dim3 block(128), grid((h->nx + 127) / 128, h->ny, h->nz);
     if (h->storage == LBM_F64)
         d3_moments_kernel<double><<<grid, block, 0, h->stream>>>(
@@ -761,7 +805,7 @@ int lbm3_moments(lbm3_handle h, double* rho_dev, double* ux, double* uy, double*
     for (int a = 0; a < 4 && e == cudaSuccess; ++a)
         e = cudaMemcpyAsync(dst[a], d + a * cells, cells * sizeof(double), cudaMemcpyDeviceToHost,
                             h->stream);
-    cudaFreeAsync(d, h->stream);
+    scratch.release();
     const cudaError_t e2 = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess || e2 != cudaSuccess)
         return fail3(h, LBM_ERR_CUDA, cudaGetErrorString(e != cudaSuccess ? e : e2));
