@@ -249,6 +249,8 @@ __global__ void __launch_bounds__(kBX * kBY)
     const int x = blockIdx.x * kBX + threadIdx.x;
     const int y = blockIdx.y * kBY + threadIdx.y;
     const int z = blockIdx.z;
+    // Launched as a programmatic dependent of the previous step (no-op otherwise).
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     if (x >= g.nx || y >= g.ny) return;
     const unsigned row = static_cast<unsigned>(g.pitch);
     const unsigned slab = row * static_cast<unsigned>(g.ny);
@@ -282,6 +284,7 @@ __global__ void __launch_bounds__(kBX * kBY)
     d3_collide<T, VAR>(f, chi, k);
 #pragma unroll
     for (int i = 0; i < kQ; ++i) dst[plane_off<NARROW>(i, g.plane, o)] = f[i];
+    asm volatile("griddepcontrol.launch_dependents;");
 }
 
 // Store population i of cell (x, y, z) in the slot its first pull reads, and zero in the
@@ -562,10 +565,19 @@ D3Const<CT> make_const(const lbm3_ctx& h) {
     return k;
 }
 
+// One step; dependent: as a programmatic dependent of the step before it in the stream,
+// so that its launch overlaps that step's tail.
 template <typename T>
-cudaError_t launch_step(lbm3_ctx* h) {
-    const dim3 block(kBX, kBY);
-    const dim3 grid((h->nx + kBX - 1) / kBX, (h->ny + kBY - 1) / kBY, h->nz);
+cudaError_t launch_step(lbm3_ctx* h, bool dependent) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.blockDim = dim3(kBX, kBY);
+    cfg.gridDim = dim3((h->nx + kBX - 1) / kBX, (h->ny + kBY - 1) / kBY, h->nz);
+    cfg.stream = h->stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = dependent ? 1 : 0;
     const T* s = static_cast<const T*>(h->buf[h->cur]);
     T* d = static_cast<T*>(h->buf[h->cur ^ 1]);
     const D3Const<T> k = make_const<T>(*h);
@@ -575,13 +587,10 @@ cudaError_t launch_step(lbm3_ctx* h) {
     const bool narrow = static_cast<unsigned long long>(kQ) * h->g.plane < (1ull << 32);
 #define LBM3_CASE(V, B)                                                                          \
     if (h->variant == V && h->bc == B) {                                                         \
-        if (narrow)                                                                              \
-            d3_step_kernel<T, V, B, true><<<grid, block, 0, h->stream>>>(s, d, h->g, k, cx, cy, \
-                                                                          cz);                   \
-        else                                                                                     \
-            d3_step_kernel<T, V, B, false><<<grid, block, 0, h->stream>>>(s, d, h->g, k, cx, cy, \
-                                                                           cz);                  \
-        return cudaGetLastError();                                                               \
+        return narrow ? cudaLaunchKernelEx(&cfg, d3_step_kernel<T, V, B, true>, s, d, h->g, k, cx, \
+                                           cy, cz)                                               \
+                      : cudaLaunchKernelEx(&cfg, d3_step_kernel<T, V, B, false>, s, d, h->g, k,  \
+                                           cx, cy, cz);                                          \
     }
     LBM3_CASE(LBM_SPONGE_NONE, LBM_BC_DIRICHLET_EQ)
     LBM3_CASE(LBM_SPONGE_I, LBM_BC_DIRICHLET_EQ)
@@ -775,7 +784,8 @@ int lbm3_step(lbm3_handle h, int nsteps) {
     if (nsteps < 0) return fail3(h, LBM_ERR_ARG, "nsteps < 0");
     if (!h->ready) return fail3(h, LBM_ERR_STATE, "step before lbm3_init_equilibrium");
     for (int t = 0; t < nsteps; ++t) {
-        const cudaError_t e = h->storage == LBM_F64 ? launch_step<double>(h) : launch_step<float>(h);
+        const cudaError_t e = h->storage == LBM_F64 ? launch_step<double>(h, t > 0)
+                                                        : launch_step<float>(h, t > 0);
         if (e != cudaSuccess) return fail3(h, LBM_ERR_CUDA, cudaGetErrorString(e));
         h->cur ^= 1;
         ++h->time;
