@@ -172,13 +172,16 @@ cudaError_t with_tile_kernel(int variant, int bc, F f) {
     return cudaErrorInvalidValue;
 }
 
-// Raise the kernel's dynamic shared-memory limit to what the tile needs (outside any
-// stream capture, before its first launch).
+// Raise the kernel's dynamic shared-memory limit (outside any stream capture, before its
+// first launch).  The limit is the kernel's, not the handle's: it is the same for
+// every tile, so that a handle with small tiles does not lower it for one with large.
+constexpr int kTileSmem = 96 * 1024;
 template <typename T>
 cudaError_t prepare_tile_t(int variant, int bc, const TileShape& t) {
+    if (tile_smem_bytes(t) > kTileSmem) return cudaErrorInvalidValue;
     const auto raise = [&](auto kernel) {
         return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    static_cast<int>(tile_smem_bytes(t)));
+                                    kTileSmem);
     };
     const cudaError_t e = with_tile_kernel<T, 1>(variant, bc, raise);
     return e == cudaSuccess ? with_tile_kernel<T, 2>(variant, bc, raise) : e;

@@ -68,3 +68,15 @@ def test_tiles_equal_a_launch_per_step(shape, bc, storage):
         steps = [2, 3, 1, 7, 130]  # single launches, replayed graphs and what they leave over
         a = _state(w, storage, True, steps)
         np.testing.assert_array_equal(a, _state(w, storage, False, steps), err_msg=variant)
+
+
+def test_a_smaller_lattice_made_later_leaves_a_larger_one_its_tiles():
+    """The kernels' shared-memory limit belongs to the process, not to a handle."""
+    from paper_1203_6350_gb300 import lbm
+
+    big, small = (_workload(n, n, "dirichlet", "II", 5, seed=n) for n in (200, 64))
+    with lbm.Lattice.from_workload(big) as a, lbm.Lattice.from_workload(small) as b:
+        b.step(12)
+        a.step(12)
+        got = a.get_state()[0]
+    np.testing.assert_array_equal(got, _state(big, "f32", False, [12]))
