@@ -15,7 +15,8 @@ __host__ __device__ constexpr int march_per_sm(int nl) { return nl == 2 ? 16 : 1
 constexpr int kMarchChunks = 17;              // chunks of four elements per staged plane-row
 constexpr int kMarchStage = 9 * kMarchChunks; // chunks per ring slot
 constexpr int kMarchRow = 4 * kMarchChunks;   // elements per staged plane-row
-constexpr int kMarchSlots = 3;                // ring slots: two rows ahead of the walk
+constexpr int kMarchSlots = 3;                // ring slots: two rows ahead of the walk (4096^2 FP32
+                                              // on the prototype: 2 slots 180 GLUPS, 3 209, 4 206, 5 145)
 constexpr int kMarchMaxSeg = 64;              // rows of a segment at most
 
 // How a launch is cut (march_rectangle, march_cut): columns [s0, s1) of strips and rows
@@ -70,7 +71,8 @@ inline int march_cut(MarchGrid& m, int ny, int seg) {
 
 // The shortest segments whose blocks (blocks(seg) of them) fit the device's slots k
 // times, for the smallest k that keeps them within kMarchMaxSeg rows: the last wave is
-// then nearly full, and few rows are computed twice.
+// then nearly full, and few rows are computed twice.  2048^2 FP32, three levels: 189 GLUPS
+// with segments of 16 rows, 219 fitted (the two-step tiles: 129).
 template <typename F>
 inline int march_segment(int nl, int sms, F blocks) {
     const long long slots = static_cast<long long>(sms) * march_per_sm(nl);
