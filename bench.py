@@ -1093,8 +1093,9 @@ def run_batched(steps: int = 1000, warmup: int = 64, count: int = 256):
         "lattices": count, "cells": cells, "steps": steps, "tile": list(cfg["tile"]),
         "cells_per_thread": cfg["cells"], "steps_per_launch": cfg["steps_per_launch"],
         "kernel": {(1, 1): "batch_step_kernel<float>", (2, 1): "batch_step2_kernel<float>",
-                   (2, 2): ("batch_tb2_tma_kernel<variant> (Dirichlet instances staged by TMA)"
-                            if staged else "batch_tb2_kernel<float>")
+                   (2, 2): ("march_batch_kernel<float, variant, 3> (large enough Dirichlet "
+                            "lattices; otherwise " + ("batch_tb2_tma_kernel<variant>)" if staged
+                                                      else "batch_tb2_kernel<float>)"))
                    }[(cfg["cells"], cfg["steps_per_launch"])],
         "mlups": cells * steps / t_batch / 1e6,
         "plain_loop_mlups": cells * steps / t_plain / 1e6,
