@@ -300,9 +300,6 @@ bool march_pays(const lbm_ctx* h, size_t l2) {
     return h->storage == LBM_F32 && 2 * h->buf_bytes > l2;
 }
 
-// Steps of one marching launch.  Results do not depend on it: FP32 levels are
-// what a store would hold, and 16-bit levels are rounded where one (spl = 1) or
-// two steps per launch (spl = 2) round them.
 // Small lattices take several steps per launch on tiles of 32-column regions.  Up to
 // 128^2 cells six steps on tiles of 4 rows (64^2 0.87 us per step, 100^2 0.89; with 8
 // steps 0.90, 0.93); up to 226^2 four steps on tiles of 16 rows (200^2 1.31 us; with six
@@ -363,6 +360,9 @@ void prepare_tiles(lbm_ctx* h) {
 }
 
 bool marching(const lbm_ctx* h) { return h->march && h->cpt == 2; }
+// Steps of one marching launch.  Results do not depend on it: FP32 levels are
+// what a store would hold, and 16-bit levels are rounded where one (spl = 1) or
+// two steps per launch (spl = 2) round them.
 int march_steps(const lbm_ctx* h) { return h->storage != LBM_F32 && h->spl == 2 ? 2 : 3; }
 
 cudaError_t launch_march(lbm_ctx* h, const void* src, void* dst, cudaStream_t st, bool pdl) {
@@ -618,8 +618,8 @@ int lbm_create(int nx, int ny, lbm_storage storage, double rho0, double ux0, dou
         if (!std::strcmp(c, "1")) h->spl = 1;
     }
     if (bc == LBM_BC_CHANNEL) h->spl = 1;  // the two-step tiles have no channel edges
-    // FP32 Dirichlet lattices whose state exceeds four times L2 stage the
-    // two-step tiles' input by TMA: measured 2-8 % ahead of plain loads from
+    // Where they run (the marching kernels come first), two-step tiles of FP32 Dirichlet
+    // lattices whose state exceeds four times L2 stage their input by TMA: measured 2-8 % ahead of plain loads from
     // 4096^2 up, 3 % behind at 2048^2 (LBM_TMA=0 or 1 overrides the choice).
     // 16-bit storage can be staged too (LBM_TMA=1), measured level with plain loads.
     const char* tma_env = std::getenv("LBM_TMA");
