@@ -384,7 +384,7 @@ __global__ void d3_moments_kernel(const T* __restrict__ src, D3Geom g, double rh
     const double r = rho0 + m[0];
     const size_t c = (static_cast<size_t>(z) * g.ny + y) * g.nx + x;
     rho[c] = m[0];
-    const lbm::Reciprocal inv = lbm::reciprocal(r, static_cast<float>(r));
+    const lbm::Reciprocal inv = lbm::reciprocal(r);
     ux[c] = lbm::quotient(rho0 * ux0 + m[1], inv, isfinite(m[1]));
     uy[c] = lbm::quotient(rho0 * uy0 + m[2], inv, isfinite(m[2]));
     uz[c] = lbm::quotient(rho0 * uz0 + m[3], inv, isfinite(m[3]));

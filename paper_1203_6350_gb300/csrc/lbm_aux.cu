@@ -196,8 +196,8 @@ __device__ __forceinline__ void cell_moments(const PlanePtrs<T>& src, const Geom
 // with divisions, 472 us now (2.1 TB/s; floor 150 us), the same bits.
 template <typename T, int BC>
 __global__ void __launch_bounds__(256)
-    moments_kernel(PlanePtrs<T> src, Geometry g, BaseState b, float rho0_f, double* rho_dev,
-                   double* ux, double* uy, LineSource ls) {
+    moments_kernel(PlanePtrs<T> src, Geometry g, BaseState b, double* rho_dev, double* ux,
+                   double* uy, LineSource ls) {
     using CT = typename Codec<T>::CT;
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(256)
         if (ux) ux[c] = __fma_rn(b.rho0, b.ux0, jx) / rho;
         if (uy) uy[c] = __fma_rn(b.rho0, b.uy0, jy) / rho;
     } else {
-        const Reciprocal inv = reciprocal(rho, rho0_f + r);
+        const Reciprocal inv = reciprocal(rho);
         if (ux) ux[c] = quotient(__fma_rn(b.rho0, b.ux0, widen(jx)), inv, isfinite(jx));
         if (uy) uy[c] = quotient(__fma_rn(b.rho0, b.uy0, widen(jy)), inv, isfinite(jy));
     }
@@ -270,13 +270,12 @@ cudaError_t moments_t(const void* src, const Geometry& g, const BaseState& b, in
                       double* ux, double* uy, cudaStream_t st, const LineSource& ls) {
     const dim3 block(128, 2), grid((g.nx + 127) / 128, (g.ny + 1) / 2);
     const PlanePtrs<T> s = plane_ptrs<T>(const_cast<void*>(src), g.plane);
-    const float rho0_f = static_cast<float>(b.rho0);
     if (bc == kPeriodic)
-        moments_kernel<T, kPeriodic><<<grid, block, 0, st>>>(s, g, b, rho0_f, r, ux, uy, ls);
+        moments_kernel<T, kPeriodic><<<grid, block, 0, st>>>(s, g, b, r, ux, uy, ls);
     else if (bc == kChannel)
-        moments_kernel<T, kChannel><<<grid, block, 0, st>>>(s, g, b, rho0_f, r, ux, uy, ls);
+        moments_kernel<T, kChannel><<<grid, block, 0, st>>>(s, g, b, r, ux, uy, ls);
     else
-        moments_kernel<T, kDirichlet><<<grid, block, 0, st>>>(s, g, b, rho0_f, r, ux, uy, ls);
+        moments_kernel<T, kDirichlet><<<grid, block, 0, st>>>(s, g, b, r, ux, uy, ls);
     return cudaGetLastError();
 }
 

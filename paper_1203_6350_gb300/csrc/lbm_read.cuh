@@ -18,19 +18,28 @@ __device__ __forceinline__ double widen(float v) {
 }
 __device__ __forceinline__ double widen(double v) { return v; }
 
+// The float nearest to v towards zero, in integer instructions (v in the range of reciprocal).
+__device__ __forceinline__ float narrow(double v) {
+    const unsigned hi = static_cast<unsigned>(__double2hiint(v));
+    const unsigned t = (hi & 0x7fffffffu) - 0x38000000u;
+    return __uint_as_float((hi & 0x80000000u) |
+                           __funnelshift_l(static_cast<unsigned>(__double2loint(v)), t, 3));
+}
+
 // 1/rho for quotients by one rho: an approximation y with relative error below 2^-42,
-// from the FP32 reciprocal by one Newton step (two FP64 instructions).
+// from the FP32 reciprocal of rho cut to FP32 (each 2^-23 off at most) by one Newton step
+// (two FP64 instructions).  It is rho itself that is cut: an FP32 sum of its terms loses all
+// digits where they cancel, near vacuum.
 struct Reciprocal {
     double rho, y;
-    bool ok;  // rho and its FP32 image are in the range where y is that good
+    bool ok;  // |rho| in [2^-60, 2^60), where y is that good
 };
-// rho_f: rho to FP32 accuracy.
-__device__ __forceinline__ Reciprocal reciprocal(double rho, float rho_f) {
+__device__ __forceinline__ Reciprocal reciprocal(double rho) {
     Reciprocal r;
     r.rho = rho;
-    const float a = fabsf(rho_f);
-    r.ok = a > 1e-18f && a < 1e18f;  // (false for NaN)
-    const double y0 = widen(rcp_eq(r.ok ? rho_f : 1.0f));
+    const unsigned t = static_cast<unsigned>(__double2hiint(rho)) & 0x7fffffffu;
+    r.ok = t - 0x3c300000u < 0x07800000u;  // (false for infinities and NaN)
+    const double y0 = widen(rcp_eq(r.ok ? narrow(rho) : 1.0f));
     r.y = __fma_rn(__fma_rn(-rho, y0, 1.0), y0, y0);
     return r;
 }
