@@ -385,9 +385,9 @@ __global__ void d3_moments_kernel(const T* __restrict__ src, D3Geom g, double rh
     const size_t c = (static_cast<size_t>(z) * g.ny + y) * g.nx + x;
     rho[c] = m[0];
     const lbm::Reciprocal inv = lbm::reciprocal(r);
-    ux[c] = lbm::quotient(rho0 * ux0 + m[1], inv, isfinite(m[1]));
-    uy[c] = lbm::quotient(rho0 * uy0 + m[2], inv, isfinite(m[2]));
-    uz[c] = lbm::quotient(rho0 * uz0 + m[3], inv, isfinite(m[3]));
+    ux[c] = lbm::quotient(rho0 * ux0 + m[1], inv);
+    uy[c] = lbm::quotient(rho0 * uy0 + m[2], inv);
+    uz[c] = lbm::quotient(rho0 * uz0 + m[3], inv);
 }
 
 constexpr int kD3Diag = 7;           // sums of lbm3_diagnostics

@@ -213,8 +213,8 @@ __global__ void __launch_bounds__(256)
         if (uy) uy[c] = __fma_rn(b.rho0, b.uy0, jy) / rho;
     } else {
         const Reciprocal inv = reciprocal(rho);
-        if (ux) ux[c] = quotient(__fma_rn(b.rho0, b.ux0, widen(jx)), inv, isfinite(jx));
-        if (uy) uy[c] = quotient(__fma_rn(b.rho0, b.uy0, widen(jy)), inv, isfinite(jy));
+        if (ux) ux[c] = quotient(__fma_rn(b.rho0, b.ux0, widen(jx)), inv);
+        if (uy) uy[c] = quotient(__fma_rn(b.rho0, b.uy0, widen(jy)), inv);
     }
 }
 

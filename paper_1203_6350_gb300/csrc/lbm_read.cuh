@@ -46,9 +46,14 @@ __device__ __forceinline__ Reciprocal reciprocal(double rho) {
 // a / rho: the quotient a y corrected by its exact remainder (P. Markstein, IBM J. Res.
 // Dev. 34, 1990), three FP64 instructions; the remainder of a quotient good to 2^-42 is
 // itself good to 2^-53, so the result is the correctly rounded quotient but for ties
-// within 2^-30 of an ulp.  Infinities and NaN, and rho out of range, take the division.
-__device__ __forceinline__ double quotient(double a, const Reciprocal& r, bool a_finite) {
-    if (!r.ok || !a_finite) return a / r.rho;
+// within 2^-30 of an ulp.  A zero keeps its sign.  Infinities, NaN and numbers outside
+// [2^-900, 2^900), whose remainder may be neither exact nor finite, and rho out of range,
+// take the division.
+__device__ __forceinline__ double quotient(double a, const Reciprocal& r) {
+    const unsigned t = static_cast<unsigned>(__double2hiint(a)) & 0x7fffffffu;
+    if (!r.ok) return a / r.rho;
+    if (t - 0x07b00000u >= 0x70800000u)
+        return (t | static_cast<unsigned>(__double2loint(a))) == 0u ? a * r.y : a / r.rho;
     const double q = a * r.y;
     return __fma_rn(__fma_rn(-r.rho, q, a), r.y, q);
 }

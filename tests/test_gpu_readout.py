@@ -56,3 +56,36 @@ def test_velocity_where_the_density_cancels(rho0, u0):
         fma = [float(Fraction(rho0) * Fraction(u0) + Fraction(float(v))) if np.isfinite(v)
                else float(v) for v in b]  # rho0 u0 + j', rounded once
         _check(uy[1], np.array(fma), rho0 + dr[1])
+
+
+def _d3_state(lat, shape, planes):
+    """The populations of a periodic D3Q15 state that varies along x only."""
+    nx, ny, nz = shape
+    buf, _ = lat.get_state()
+    s = np.zeros((15, nz, ny, buf.nbytes // (15 * nz * ny * 8)))
+    for i, v in planes.items():
+        s[i, :, :, :nx] = v
+    lat.set_state(s.view(np.uint8).ravel(), 0)
+
+
+def _d3_fields(rho0, planes):
+    """(rho', u_y) along x of an FP64 state given by its populations (3: c = +y, 4: -y)."""
+    from paper_1203_6350_gb300 import lbm
+
+    shape = (len(planes[0]), 3, 2)
+    with lbm.Lattice3(*shape, "f64", rho0, (0.0, 0.0, 0.0), 1.9, bc="periodic") as lat:
+        lat.init_equilibrium(np.full(shape[::-1], rho0), 0.0, 0.0, 0.0)
+        _d3_state(lat, shape, planes)
+        rho, ux, uy, uz = lat.moments()
+        return rho[1, 1], ux[1, 1], uy[1, 1], uz[1, 1]
+
+
+@pytest.mark.parametrize("rho0", [1.0, 3e-18, 5e17])
+def test_quotients_of_huge_and_tiny_momenta(rho0):
+    """FP64 momenta whose quotient overflows, or whose remainder underflows."""
+    j = np.array([0.0, 1.0, -0.3, 1e270, -1e270, 1e300, 1.7e308, -1.7e308, 1e-270, 1e-290,
+                  -1e-300, 3e-308, 5e-324, -1e-320])
+    rho, ux, uy, uz = _d3_fields(rho0, {0: -j, 3: j})  # the rest population takes it back
+    np.testing.assert_array_equal(rho, np.zeros_like(j))
+    assert not ux.any() and not uz.any()
+    _check(uy, j, np.full_like(j, rho0))
