@@ -344,6 +344,21 @@ __global__ void __launch_bounds__(128)
     }
 }
 
+// Population i that the pull at a cell reads (0 from outside a Dirichlet lattice).
+template <typename T>
+__device__ __forceinline__ double d3_pulled(const T* __restrict__ src, const D3Geom& g, int bc,
+                                            int i, int x, int y, int z) {
+    int sx = x - d3cx(i), sy = y - d3cy(i), sz = z - d3cz(i);
+    if (bc == LBM_BC_PERIODIC) {
+        sx = wrap(sx, g.nx);
+        sy = wrap(sy, g.ny);
+        sz = wrap(sz, g.nz);
+    }
+    if (sx < 0 || sx >= g.nx || sy < 0 || sy >= g.ny || sz < 0 || sz >= g.nz) return 0.0;
+    return lbm::widen(src[static_cast<size_t>(i) * g.plane +
+                          (static_cast<unsigned>(sz) * g.ny + sy) * g.pitch + sx]);
+}
+
 // Deviations (rho', j - rho0 u0) of the pulled (pre-collision) state at a cell.
 template <typename T>
 __device__ __forceinline__ void d3_pulled_moments(const T* __restrict__ src, const D3Geom& g,
@@ -351,21 +366,22 @@ __device__ __forceinline__ void d3_pulled_moments(const T* __restrict__ src, con
     m[0] = m[1] = m[2] = m[3] = 0.0;
 #pragma unroll
     for (int i = 0; i < kQ; ++i) {
-        int sx = x - d3cx(i), sy = y - d3cy(i), sz = z - d3cz(i);
-        double v = 0.0;
-        if (bc == LBM_BC_PERIODIC) {
-            sx = wrap(sx, g.nx);
-            sy = wrap(sy, g.ny);
-            sz = wrap(sz, g.nz);
-        }
-        if (sx >= 0 && sx < g.nx && sy >= 0 && sy < g.ny && sz >= 0 && sz < g.nz)
-            v = lbm::widen(src[static_cast<size_t>(i) * g.plane +
-                               (static_cast<unsigned>(sz) * g.ny + sy) * g.pitch + sx]);
+        const double v = d3_pulled(src, g, bc, i, x, y, z);
         m[0] += v;
         if (d3cx(i) != 0) m[1] += d3cx(i) * v;
         if (d3cy(i) != 0) m[2] += d3cy(i) * v;
         if (d3cz(i) != 0) m[3] += d3cz(i) * v;
     }
+    // An infinite population makes its product with a zero component NaN, so that a cell
+    // of a state that has overflowed reports no finite velocity.
+    if (!isfinite(m[0]))
+#pragma unroll 1
+        for (int i = 0; i < kQ; ++i) {
+            const double v = d3_pulled(src, g, bc, i, x, y, z);
+            m[1] += 0.0 * v;
+            m[2] += 0.0 * v;
+            m[3] += 0.0 * v;
+        }
 }
 
 // rho' and u of the pulled (pre-collision) state, FP64 [nz][ny][nx].

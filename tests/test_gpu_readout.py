@@ -89,3 +89,22 @@ def test_quotients_of_huge_and_tiny_momenta(rho0):
     np.testing.assert_array_equal(rho, np.zeros_like(j))
     assert not ux.any() and not uz.any()
     _check(uy, j, np.full_like(j, rho0))
+
+
+def test_an_infinite_population_leaves_no_velocity():
+    """An overflowed cell of a 3-D state: the products of an infinite population with the
+    zero components of its velocity are NaN, and so is u.  Finite populations whose sum
+    overflows still have the quotient of their momentum."""
+    inf, big = np.inf, 1.2e308
+    rest = np.array([inf, -inf, np.nan, 0.0, 0.0, 0.0, inf, 0.0, big, big])
+    plus = np.array([0.0, 0.0, 0.0, inf, 0.0, np.nan, -inf, inf, 0.0, big])
+    minus = np.array([0.0, 0.0, 0.0, 0.0, -inf, 0.0, 0.0, inf, 0.0, 0.0])
+    rho, ux, uy, uz = _d3_fields(1.0, {0: rest, 3: plus, 4: minus})
+    with np.errstate(all="ignore"):
+        np.testing.assert_array_equal(rho, rest + plus + minus)
+        want = np.full(rest.shape, np.nan)
+        want[-2:] = plus[-2:] / (1.0 + rho[-2:])
+    np.testing.assert_array_equal(uy, want)
+    want[-2:] = 0.0
+    np.testing.assert_array_equal(ux, want)
+    np.testing.assert_array_equal(uz, want)
