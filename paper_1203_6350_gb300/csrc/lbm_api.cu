@@ -793,10 +793,11 @@ int lbm_step(lbm_handle h, int nsteps) {
             }
         }
     }
-    // the channel issues at most kGraphChunk launches per source table
+    // the channel's source table holds kGraphChunk steps; a graph's steps are as many of
+    // them as make whole launches
     while (nsteps > 0) {
         const bool channel = h->bc == LBM_BC_CHANNEL;
-        const int chunk = channel && nsteps > kGraphChunk ? kGraphChunk : nsteps;
+        const int chunk = channel && nsteps > graph_steps ? graph_steps : nsteps;
         if (channel) {
             e = launch_source_table(h, h->stream, chunk);
             if (e != cudaSuccess) return cuda_fail(h, e, "lbm_step source table");
