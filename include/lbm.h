@@ -155,12 +155,18 @@ int lbm_init_pulse(lbm_handle h, double eps, double half_width, double x0, doubl
  * 226 x 226 cells) up to six, on tiles in shared memory; the results are those of
  * the launches that lbm_set_steps_per_launch describes, bit for bit, and
  * lbm_set_steps_per_launch or lbm_set_tma_staging (or their environment
- * variables) select those launches instead. */
+ * variables) select those launches instead.
+ *
+ * On a stream under capture the steps become part of the caller's graph.  A
+ * graph whose nsteps are a multiple of two (of four, where
+ * lbm_steps_per_launch is 2) ends in the buffer it began with, so each replay
+ * takes nsteps steps more; the handle's own count (lbm_time) knows only the
+ * captured call. */
 int lbm_step(lbm_handle h, int nsteps);
 
 /* Step kernels that lbm_step(h, nsteps) launches as the handle is set up now,
- * those of replayed graphs included (LBM_ERR_ARG for a NULL handle or
- * nsteps < 0).  No CUDA call. */
+ * on a stream that is not under capture, those of replayed graphs included
+ * (LBM_ERR_ARG for a NULL handle or nsteps < 0).  No CUDA call. */
 int lbm_step_launches(lbm_handle h, int nsteps);
 
 /* Fields at the current time: rho_dev = rho - rho0, ux, uy (FP64 [ny][nx];

@@ -384,15 +384,17 @@ cudaError_t launch_march(lbm_ctx* h, const void* src, void* dst, cudaStream_t st
     }
 }
 
-// Advance `left` steps' first launch from src to dst; *taken receives its steps.
-cudaError_t launch_steps(lbm_ctx* h, const void* src, void* dst, int left, cudaStream_t st,
-                         bool pdl, long long t_off, int* taken) {
-    if (marching(h) && left >= march_steps(h)) {
+// Advance the first launch of `left` steps from src to dst; *taken receives its steps.  Only
+// the first `grouped` of them may go to the marching and the tile kernels.
+cudaError_t launch_steps(lbm_ctx* h, const void* src, void* dst, int left, int grouped,
+                         cudaStream_t st, bool pdl, long long t_off, int* taken) {
+    const int g = grouped < left ? grouped : left;
+    if (marching(h) && g >= march_steps(h)) {
         *taken = march_steps(h);
         return launch_march(h, src, dst, st, pdl);
     }
-    if (tiled(h) && left >= 2) {
-        *taken = tile_steps(h, left);
+    if (tiled(h) && g >= 2) {
+        *taken = tile_steps(h, g);
         return launch_tile(h, src, dst, *taken, st, pdl, t_off);
     }
     *taken = h->spl == 2 && left >= 2 ? 2 : 1;
@@ -405,6 +407,16 @@ cudaError_t launch_steps(lbm_ctx* h, const void* src, void* dst, int left, cudaS
 int graph_chunk(const lbm_ctx* h) {
     if (tiled(h)) return h->tile_levels == 6 ? 60 : kGraphChunk;  // 10 or 16 launches
     return marching(h) && march_steps(h) == 3 ? kMarchChunk : kGraphChunk;
+}
+
+// How many of nsteps steps on a captured stream may go to the marching and the tile kernels.
+// A program replays its graph, and each replay goes on from where the last one ended only
+// if the graph returns to the buffer it began with.  Whether it does stays what it is with
+// the launches that the handle's settings name: groups of steps that are an even number of
+// launches in either way (twelve steps are 4 marching launches of three, 6 of two, or 12
+// or 6 named ones).
+int grouped_under_capture(const lbm_ctx* h, int nsteps) {
+    return nsteps - nsteps % (tiled(h) ? 2 * h->tile_levels : 12);
 }
 
 // Tensor maps, persistent grid and error flag of the TMA two-step kernel;
@@ -472,7 +484,8 @@ cudaError_t ensure_graph(lbm_ctx* h, int parity) {
     if (h->bc == LBM_BC_CHANNEL) e = launch_source_table(h, h->capture_stream, chunk);
     int c = parity;
     for (int t = 0, n = 0; t < chunk && e == cudaSuccess; t += n) {
-        e = launch_steps(h, h->buf[c], h->buf[1 - c], chunk - t, h->capture_stream, t > 0, t, &n);
+        e = launch_steps(h, h->buf[c], h->buf[1 - c], chunk - t, chunk - t, h->capture_stream, t > 0,
+                         t, &n);
         c = 1 - c;
     }
     if (e == cudaSuccess && h->bc == LBM_BC_CHANNEL) {  // the line source's clock
@@ -778,21 +791,25 @@ int lbm_step(lbm_handle h, int nsteps) {
     cudaError_t e = cudaSuccess;
     const bool pdl = h->launch_mode != kLaunchPlain;
     const int graph_steps = graph_chunk(h);
-    if (h->launch_mode == kLaunchGraph && nsteps >= graph_steps) {
+    const bool graph = h->launch_mode == kLaunchGraph && nsteps >= graph_steps;
+    bool capturing = false;
+    if (graph || marching(h) || tiled(h)) {
         cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
         e = cudaStreamIsCapturing(h->stream, &cs);
         if (e != cudaSuccess) return cuda_fail(h, e, "cudaStreamIsCapturing");
-        if (cs == cudaStreamCaptureStatusNone) {
-            e = ensure_graph(h, h->cur);
-            if (e != cudaSuccess) return cuda_fail(h, e, "lbm_step graph build");
-            while (nsteps >= graph_steps) {
-                e = cudaGraphLaunch(h->graph[h->cur], h->stream);
-                if (e != cudaSuccess) return cuda_fail(h, e, "lbm_step graph launch");
-                h->time += graph_steps;  // an even number of launches leaves cur unchanged
-                nsteps -= graph_steps;
-            }
+        capturing = cs != cudaStreamCaptureStatusNone;
+    }
+    if (graph && !capturing) {
+        e = ensure_graph(h, h->cur);
+        if (e != cudaSuccess) return cuda_fail(h, e, "lbm_step graph build");
+        while (nsteps >= graph_steps) {
+            e = cudaGraphLaunch(h->graph[h->cur], h->stream);
+            if (e != cudaSuccess) return cuda_fail(h, e, "lbm_step graph launch");
+            h->time += graph_steps;  // an even number of launches leaves cur unchanged
+            nsteps -= graph_steps;
         }
     }
+    int grouped = capturing ? grouped_under_capture(h, nsteps) : nsteps;
     // the channel's source table holds kGraphChunk steps; a graph's steps are as many of
     // them as make whole launches
     while (nsteps > 0) {
@@ -805,12 +822,13 @@ int lbm_step(lbm_handle h, int nsteps) {
         int issued = 0;
         while (issued < chunk) {
             int n = 0;
-            e = launch_steps(h, h->buf[h->cur], h->buf[1 - h->cur], chunk - issued, h->stream, pdl,
-                             issued, &n);
+            e = launch_steps(h, h->buf[h->cur], h->buf[1 - h->cur], chunk - issued, grouped,
+                             h->stream, pdl, issued, &n);
             if (e != cudaSuccess) return cuda_fail(h, e, "lbm_step launch");
             h->cur = 1 - h->cur;
             h->time += n;
             issued += n;
+            grouped -= n;
         }
         nsteps -= chunk;
         if (channel) {  // the line source's clock
