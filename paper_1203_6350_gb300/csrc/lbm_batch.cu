@@ -734,6 +734,8 @@ struct lbm_batch_ctx {
         std::vector<lbm::MarchItem> items;
     };
     bool march = false;
+    bool captured = false;  // a captured lbm_batch_step may have been replayed: the device's
+                            // step counter may be ahead of `step`
     int sms = 0;
     std::vector<MarchGroup> march_groups;
     lbm::MarchBatch march_params;  // the launch being built
@@ -1495,11 +1497,13 @@ int lbm_batch_step(lbm_batch b, int nsteps) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     e = cudaStreamIsCapturing(b->stream, &cs);
     if (e != cudaSuccess) return bfail(b, LBM_ERR_CUDA, "cudaStreamIsCapturing");
-    // Marching launches carry the instances' buffers, as the host knows them, in their
-    // parameters; a captured stream is replayed with others, so it keeps to the kernels that
-    // read them on the device.
+    // Marching launches carry the instances' buffers and their places in the budgets, as the
+    // host knows them, in their parameters.  A captured stream is replayed with others, and
+    // once it has been the host does not know them, so such a batch keeps to the kernels
+    // that read them on the device.
+    if (cs != cudaStreamCaptureStatusNone) b->captured = true;
     int step_off = 0, launch_off = 0;
-    for (bool march = b->march && cs == cudaStreamCaptureStatusNone;
+    for (bool march = b->march && !b->captured;
          march && nsteps >= march_levels(b);) {
         const int d = march_levels(b);
         e = launch_march(b, b->step + step_off, d, launch_off > 0, &march);

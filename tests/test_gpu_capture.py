@@ -65,3 +65,34 @@ def test_replays_of_captured_steps_go_on(shape, bc, steps, storage):
             lat.step(steps)
         want, _ = lat.get_state()
     np.testing.assert_array_equal(got, want)
+
+
+def test_a_batch_steps_on_after_replays(monkeypatch):
+    """Replays advance the device's step counter alone, and a budget ends by that counter."""
+    import torch
+    from paper_1203_6350_gb300.batch import Batch
+
+    works = [_workload(420, 400, "dirichlet", seed=1), _workload(430, 390, "dirichlet", seed=2)]
+    budgets = [20, 1000]
+    config = {"cells": 2, "steps_per_launch": 2, "tile": (64, 16)}
+
+    def fields(replays):
+        stream = torch.cuda.Stream()
+        with Batch("f32", stream=stream, config=config) as b:
+            ids = [b.add_workload(w, steps=n) for w, n in zip(works, budgets)]
+            b.step(4)
+            if replays:  # 4 steps, then 3 x 4 replayed, then 12 more
+                graph = _graph(stream, lambda: b.step(4))
+                with torch.cuda.stream(stream):
+                    for _ in range(3):
+                        graph.replay()
+                b.step(12)
+            else:
+                b.step(24)
+            return [b.moments(i) for i in ids]
+
+    monkeypatch.delenv("LBM_BATCH_TMA", raising=False)
+    got = fields(True)
+    monkeypatch.setenv("LBM_BATCH_TMA", "1")  # the tile kernels throughout
+    for a, b in zip(got, fields(False)):
+        np.testing.assert_array_equal(a, b)
