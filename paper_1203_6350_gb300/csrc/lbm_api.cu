@@ -305,7 +305,6 @@ bool march_pays(const lbm_ctx* h, size_t l2) {
 // steps 0.90, 0.93); up to 226^2 four steps on tiles of 16 rows (200^2 1.31 us; with six
 // and 10 rows 1.87).  Above, a launch per step is level or faster (300^2 1.97 us
 // against 2.37, 800 x 200 channel 2.63 against 3.3): the cells computed twice fill the GPU.
-constexpr int kTileRegion = 32;
 void choose_tiles(lbm_ctx* h) {
     const long long cells = static_cast<long long>(h->nx) * h->ny;
     if (cells <= 128 * 128) {
@@ -333,8 +332,7 @@ cudaError_t launch_tile(lbm_ctx* h, const void* src, void* dst, int levels, cuda
     const auto launch = h->storage == LBM_F32      ? lbm::launch_tile_f32
                         : h->storage == LBM_F16DEV ? lbm::launch_tile_f16
                                                    : lbm::launch_tile_bf16;
-    return launch(src, dst, h->geo, h->k2, tx, ty, h->variant, h->bc, kTileRegion, h->tile_h,
-                  levels, st, p, ls);
+    return launch(src, dst, h->geo, h->k2, tx, ty, h->variant, h->bc, h->tile_h, levels, st, p, ls);
 }
 
 // The marching kernels' segments for the handle's layer and variant.
@@ -353,7 +351,7 @@ void prepare_tiles(lbm_ctx* h) {
     const auto prepare = h->storage == LBM_F32      ? lbm::prepare_tile_f32
                          : h->storage == LBM_F16DEV ? lbm::prepare_tile_f16
                                                     : lbm::prepare_tile_bf16;
-    if (prepare(h->variant, h->bc, kTileRegion, h->tile_h, h->tile_levels) != cudaSuccess) {
+    if (prepare(h->variant, h->bc, h->tile_h, h->tile_levels) != cudaSuccess) {
         cudaGetLastError();
         h->tile_h = 0;
     }

@@ -295,23 +295,26 @@ cudaError_t launch_march_bf16_periodic(const void* src, void* dst, const Geometr
                                    const AxisCoef<float>* ty, int variant, bool each_level, int seg,
                                    cudaStream_t st, int pdl);
 
-// Several steps (levels >= 2) per launch on tiles of h rows in regions of rw = 32 or 64
+// Several steps (levels >= 2) per launch on tiles of h rows in regions of kTileRegion
 // columns (lbm_tile.cuh), for small lattices.  prepare_tile: once per variant, before
 // the first launch, with the most levels that will be asked for.
-cudaError_t prepare_tile_f32(int variant, int bc, int rw, int h, int levels);
+constexpr int kTileRegion = 32;
+__host__ __device__ constexpr int tile_halo(int levels) { return levels / 2 * 2; }
+__host__ __device__ constexpr int tile_width(int levels) { return kTileRegion - 2 * tile_halo(levels); }
+cudaError_t prepare_tile_f32(int variant, int bc, int h, int levels);
 cudaError_t launch_tile_f32(const void* src, void* dst, const Geometry& g, const StepConst<F2>& k,
                             const AxisCoef<float>* tx, const AxisCoef<float>* ty, int variant,
-                            int bc, int rw, int h, int levels, cudaStream_t st, int pdl,
+                            int bc, int h, int levels, cudaStream_t st, int pdl,
                             const LineSource& ls);
-cudaError_t prepare_tile_f16(int variant, int bc, int rw, int h, int levels);
+cudaError_t prepare_tile_f16(int variant, int bc, int h, int levels);
 cudaError_t launch_tile_f16(const void* src, void* dst, const Geometry& g, const StepConst<F2>& k,
                             const AxisCoef<float>* tx, const AxisCoef<float>* ty, int variant,
-                            int bc, int rw, int h, int levels, cudaStream_t st, int pdl,
+                            int bc, int h, int levels, cudaStream_t st, int pdl,
                             const LineSource& ls);
-cudaError_t prepare_tile_bf16(int variant, int bc, int rw, int h, int levels);
+cudaError_t prepare_tile_bf16(int variant, int bc, int h, int levels);
 cudaError_t launch_tile_bf16(const void* src, void* dst, const Geometry& g, const StepConst<F2>& k,
                             const AxisCoef<float>* tx, const AxisCoef<float>* ty, int variant,
-                            int bc, int rw, int h, int levels, cudaStream_t st, int pdl,
+                            int bc, int h, int levels, cudaStream_t st, int pdl,
                             const LineSource& ls);
 
 // Two steps per launch with the tile's input staged by TMA (FP32, Dirichlet):
