@@ -305,12 +305,22 @@ bool march_pays(const lbm_ctx* h, size_t l2) {
 // steps 0.90, 0.93); up to 226^2 four steps on tiles of 16 rows (200^2 1.31 us; with six
 // and 10 rows 1.87).  Above, a launch per step is level or faster (300^2 1.97 us
 // against 2.37, 800 x 200 channel 2.63 against 3.3): the cells computed twice fill the GPU.
+// So they do on fewer cells where thin lattices leave most of each tile empty: the tiles
+// must fit the device at once (by their registers two blocks of 4 rows to an SM, one of
+// 16).  FP32, us per step with tiles and with a launch per step, tiles per device-full:
+// 3000 x 5 1.20 / 2.14 (0.99), 226^2 1.42 / 2.14 (0.99), but 1000 x 50 2.28 / 1.79 (1.1),
+// 50 x 1000 2.57 / 2.33 (1.2), 16000 x 1 2.83 / 1.78 (2.6), 17000 x 3 5.63 / 2.30 (4.7),
+// 1 x 16000 11.8 / 8.6 (13).
 void choose_tiles(lbm_ctx* h) {
     const long long cells = static_cast<long long>(h->nx) * h->ny;
-    if (cells <= 128 * 128) {
+    const auto fits = [&](int rows, int levels, int per_sm) {
+        const long long w = lbm::tile_width(levels);
+        return (h->nx + w - 1) / w * ((h->ny + rows - 1) / rows) <= per_sm * h->sms;
+    };
+    if (cells <= 128 * 128 && fits(4, 6, 2)) {
         h->tile_h = 4;
         h->tile_levels = 6;
-    } else if (cells <= 226 * 226) {
+    } else if (cells <= 226 * 226 && fits(16, 4, 1)) {
         h->tile_h = 16;
         h->tile_levels = 4;
     }
@@ -640,11 +650,12 @@ int lbm_create(int nx, int ny, lbm_storage storage, double rho0, double ux0, dou
     if (storage != LBM_F64 && bc == LBM_BC_DIRICHLET_EQ && want_tma)
         h->tma = setup_tma(h) == LBM_OK;
     // an environment variable that names a kernel keeps to it
-    h->march = h->cpt == 2 && !std::getenv("LBM_SPL") && !tma_env && march_pays(h, l2) &&
-               cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device) ==
-                   cudaSuccess;
+    if (h->cpt == 2 && !std::getenv("LBM_SPL") && !tma_env &&
+        cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device) == cudaSuccess) {
+        h->march = march_pays(h, l2);
+        if (h->spl == 1) choose_tiles(h);
+    }
     cut_march(h);
-    if (h->cpt == 2 && h->spl == 1 && !std::getenv("LBM_SPL") && !tma_env) choose_tiles(h);
     prepare_tiles(h);
     h->err.clear();
     set_source_shape(h);
