@@ -50,10 +50,13 @@ struct lbm_ctx {
     long long* d_time = nullptr;      // channel boundary: device copy of the step counter
     double* d_src_table = nullptr;    // channel boundary: source scales of the next kGraphChunk steps,
                                       // then their FP32 source populations (9 per step)
+    bool by_size = false;             // the kernels are chosen by size and layer, until one is asked
+                                      // for by name
     bool march = false;               // with cpt == 2: groups of march_steps() steps go to the marching
-                                      // kernels (chosen by size, until a kernel is asked for by name)
+                                      // kernels
     int march_seg = 0;                // rows of their segments
     int sms = 0;                      // multiprocessors of the device
+    size_t l2 = 0;                    // bytes of its L2 cache
     int tile_h = 0;                   // with cpt == 2: rows of the small-lattice tiles (0: not used),
     int tile_levels = 0;              // and the steps one of their launches takes at most
     bool initialised = false;
@@ -280,8 +283,9 @@ cudaError_t launch_two_steps(lbm_ctx* h, const void* src, void* dst, cudaStream_
     }
 }
 
+int march_steps(const lbm_ctx* h);
 // Whether the marching kernels are the faster ones, measured against the one-step
-// pair kernel and the tiles on square lattices (f32, ratio of throughputs):
+// pair kernel and the tiles (f32, ratio of throughputs).  By size, square lattices:
 //  - Dirichlet: 0.92 at 700^2, 1.00 at 850^2, 1.09 at 900^2, 1.05 at 1024^2, 1.9 at
 //    1300^2, 1.7 at 2048^2, 1.63 at 4096^2 (16-bit storage: 1.03 at 850^2, 1.14-1.17 at
 //    1536^2, 1.3 at 4096^2).  Fewer cells leave too few warps, each with a long walk.
@@ -290,14 +294,36 @@ cudaError_t launch_two_steps(lbm_ctx* h, const void* src, void* dst, cudaStream_
 //    rows are staged by words at the seam: 0.86 at 1150^2, but 1.12 at 1401^2 and 1.25
 //    at 2049^2 in FP32, once the state exceeds L2.
 //  - At least four strips and 64 rows, or the last strip's idle lanes and the rows
-//    computed twice eat the gain.
-bool march_pays(const lbm_ctx* h, size_t l2) {
-    if (h->nx < 240 || h->ny < 64) return false;
+//    computed twice eat the gain.  16-bit lattices that L2 holds easily need 200
+//    rows: periodic 17472 x 103 0.74, 7804 x 168 0.88, 10256 x 162 0.93, 4000 x 304 1.04,
+//    Dirichlet 18717 x 113 0.85, 11532 x 139 0.96, 2242 x 402 1.12.
+// And by the layer: a cell of the walks outside the chi = 0 rectangle costs 1.6 to 1.9 times
+// one inside (16-bit 8.8 against 4.7 ps), which the other kernels' layer cells do not.  The
+// share of such walks, up to which marching is taken:
+//  - 16-bit: 0.5 while both buffers fill 3/4 of L2 or less (bf16 1832 x 1199 0.37, 1.11;
+//    f16 1085 x 1826 0.49, 1.03; 786 x 1241 0.55, 0.95; 5724 x 415 0.65, 0.89; 850 x 1054 0.82,
+//    0.86; 1344 x 1093 0.98, 0.83), above, where the other kernels slow down, 0.85 (bf16
+//    2447 x 1187 0.73, 1.10; 2300 x 1552 0.84, 1.14; f16 8125 x 483 1, 0.96; bf16 4096^2 1, 0.97);
+//  - FP32: any (4096^2 1, 1.31; 1344 x 1093 1, 1.15), but 0.7 where the seam is staged by
+//    words (2045 x 1664 0.71, 0.98; 18899 x 156 1, 0.85).  Below 1.1 million cells a share
+//    above 0.6 costs time in FP32 too (1024^2, layer II 64 deep: 0.37, 1.07; 128 deep 0.54,
+//    511 deep 1, 0.79).
+// Without a layer every walk is the cheap one.
+bool march_pays(const lbm_ctx* h) {
+    if (h->storage == LBM_F64 || h->nx < 240 || h->ny < 64) return false;
     const long long cells = static_cast<long long>(h->nx) * h->ny;
-    if (h->bc == LBM_BC_DIRICHLET_EQ) return cells >= 800000;
-    if (h->bc != LBM_BC_PERIODIC) return false;
-    if (h->nx % 4 == 0) return cells >= 1200000;
-    return h->storage == LBM_F32 && 2 * h->buf_bytes > l2;
+    const bool f32 = h->storage == LBM_F32, periodic = h->bc == LBM_BC_PERIODIC;
+    const bool words = periodic && h->nx % 4 != 0;
+    const bool fits = 2 * h->buf_bytes / 3 <= h->l2 / 4;
+    if (h->bc == LBM_BC_CHANNEL || cells < (periodic ? 1200000 : 800000)) return false;
+    if (words && !(f32 && 2 * h->buf_bytes > h->l2)) return false;
+    if (!f32 && fits && h->ny < 200) return false;
+    if (h->variant == LBM_SPONGE_NONE || (f32 && !words)) return true;
+    const int nl = march_steps(h);
+    const lbm::MarchGrid m = lbm::march_rectangle(h->geo, h->k2, h->variant, nl);
+    const double share = 1.0 - static_cast<double>(lbm::march_fast_cells(m, nl)) /
+                                   lbm::march_cells(m, h->ny, nl);
+    return share <= (f32 ? 0.7 : fits ? 0.5 : 0.85);
 }
 
 // Small lattices take several steps per launch on tiles of 32-column regions.  Up to
@@ -325,7 +351,6 @@ void choose_tiles(lbm_ctx* h) {
         h->tile_levels = 4;
     }
 }
-int march_steps(const lbm_ctx* h);
 bool tiled(const lbm_ctx* h) { return h->tile_h > 0 && h->cpt == 2; }
 // Steps of the next launch of `left` >= 2: equal parts of at most tile_levels.
 int tile_steps(const lbm_ctx* h, int left) {
@@ -345,8 +370,9 @@ cudaError_t launch_tile(lbm_ctx* h, const void* src, void* dst, int levels, cuda
     return launch(src, dst, h->geo, h->k2, tx, ty, h->variant, h->bc, h->tile_h, levels, st, p, ls);
 }
 
-// The marching kernels' segments for the handle's layer and variant.
-void cut_march(lbm_ctx* h) {
+// Whether to march with the handle's layer and variant, and the segments.
+void choose_march(lbm_ctx* h) {
+    h->march = h->by_size && march_pays(h);
     if (!h->march) return;
     const int nl = march_steps(h);
     lbm::MarchGrid m = lbm::march_rectangle(h->geo, h->k2, h->variant, nl);
@@ -650,12 +676,12 @@ int lbm_create(int nx, int ny, lbm_storage storage, double rho0, double ux0, dou
     if (storage != LBM_F64 && bc == LBM_BC_DIRICHLET_EQ && want_tma)
         h->tma = setup_tma(h) == LBM_OK;
     // an environment variable that names a kernel keeps to it
-    if (h->cpt == 2 && !std::getenv("LBM_SPL") && !tma_env &&
-        cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device) == cudaSuccess) {
-        h->march = march_pays(h, l2);
-        if (h->spl == 1) choose_tiles(h);
-    }
-    cut_march(h);
+    h->l2 = static_cast<size_t>(l2);
+    h->by_size = h->cpt == 2 && !std::getenv("LBM_SPL") && !tma_env &&
+                 cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device) ==
+                     cudaSuccess;
+    choose_march(h);
+    if (h->by_size && h->spl == 1) choose_tiles(h);
     prepare_tiles(h);
     h->err.clear();
     set_source_shape(h);
@@ -733,7 +759,7 @@ int lbm_set_sponge(lbm_handle h, lbm_variant variant, const double* chi_x, const
     lbm::zero_run(chi_x, h->nx, h->bulk[0], h->bulk[1]);
     lbm::zero_run(chi_y, h->ny, h->bulk[2], h->bulk[3]);
     refresh_consts(h);
-    cut_march(h);
+    choose_march(h);
     prepare_tiles(h);
     const double s_nu = h->rates.s[7];
     if ((variant == LBM_SPONGE_II || variant == LBM_SPONGE_III) && chi_max > 4.0 / s_nu)
@@ -960,6 +986,7 @@ int lbm_set_cells_per_thread(lbm_handle h, int cells) {
         drop_graphs(h);  // the captured launches name the other kernel
         h->cpt = cells;
         if (cells == 1) h->spl = 1;
+        choose_march(h);  // (by the steps that 16-bit states are rounded after)
     }
     return LBM_OK;
 }
@@ -971,6 +998,7 @@ int lbm_set_steps_per_launch(lbm_handle h, int steps) {
         return fail(h, LBM_ERR_ARG, "two steps per launch needs two cells per thread");
     if (steps == 2 && h->bc == LBM_BC_CHANNEL)
         return fail(h, LBM_ERR_ARG, "two steps per launch is not available for the channel boundary");
+    h->by_size = false;
     if (steps != h->spl || h->march || h->tile_h) {
         DeviceGuard dg(h->device);
         cudaStreamSynchronize(h->stream);
@@ -1008,7 +1036,10 @@ int lbm_get_arithmetic(lbm_handle h) { return h ? h->arith : LBM_ERR_ARG; }
 int lbm_set_tma_staging(lbm_handle h, int on) {
     if (!h) return LBM_ERR_ARG;
     if (on != 0 && on != 1) return fail(h, LBM_ERR_ARG, "on must be 0 or 1");
-    if (on == (h->tma ? 1 : 0) && !h->march && !h->tile_h) return LBM_OK;
+    if (on == (h->tma ? 1 : 0) && !h->march && !h->tile_h) {
+        h->by_size = false;
+        return LBM_OK;
+    }
     if (on && h->arith == LBM_ARITH_COMPENSATED)
         return fail(h, LBM_ERR_ARG, "compensated arithmetic steps one cell, one step per launch");
     DeviceGuard dg(h->device);
@@ -1018,6 +1049,7 @@ int lbm_set_tma_staging(lbm_handle h, int on) {
     }
     cudaStreamSynchronize(h->stream);
     drop_graphs(h);  // the captured launches name the other kernel
+    h->by_size = false;
     h->march = false;
     h->tile_h = 0;
     h->tma = on == 1;

@@ -55,6 +55,14 @@ inline MarchGrid march_rectangle(const Geometry& g, const StepConst<F2>& k, int 
     return m;
 }
 
+// Cells of its strips (whole ones, so the last strip's idle lanes count), and of the rectangle.
+inline long long march_cells(const MarchGrid& m, int ny, int nl) {
+    return static_cast<long long>(m.strips) * march_width(nl) * ny;
+}
+inline long long march_fast_cells(const MarchGrid& m, int nl) {
+    return static_cast<long long>(m.s1 - m.s0) * march_width(nl) * (m.y1 - m.y0);
+}
+
 // Cut it into segments of seg rows, 5/8 as long outside the rectangle, where a row
 // costs about 1.5 times as much.  Returns the blocks.
 inline int march_cut(MarchGrid& m, int ny, int seg) {
