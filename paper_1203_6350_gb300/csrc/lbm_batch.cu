@@ -949,33 +949,52 @@ cudaError_t compute_grid(lbm_batch_ctx* b) {
 // Steps of one marching launch.
 int march_levels(const lbm_batch_ctx* b) { return b->storage == LBM_F32 ? 3 : 2; }
 
-// Whether marching launches are the faster ones for this batch (Dirichlet instances,
-// two steps per launch chosen, no environment variable that names the tile kernels'
-// loads).  Measured against the tile kernels, ratio of throughputs by count and sides:
-// FP32 256 of 64-1024 1.32, 64 of 64-1024 1.42, 32 of 64-512 1.28, 8 of 256-1024 1.52, 8 of
-// 200-300 1.13, but 32 of 64-256 0.91 and 64 of 64-128 0.91; FP16 1.14, 1.34, 1.33, 1.62,
-// 1.39, 1.29 and 1.04, 128 of 64-128 0.71.  Small instances leave a warp little but edges
-// and constants that change with every block: the line is drawn at their mean size.
-bool march_pays(const lbm_batch_ctx* b) {
+// Whether marching launches can serve this batch: Dirichlet instances, two steps per launch
+// chosen, no environment variable that names the tile kernels' loads.
+bool march_serves(const lbm_batch_ctx* b) {
     if (b->storage == LBM_F64 || b->cpt != 2 || b->spl != 2 || std::getenv("LBM_BATCH_TMA"))
         return false;
-    long long cells = 0, count = 0;
-    for (const auto& kv : b->insts) {
-        const Instance& in = kv.second;
-        if (in.bc != LBM_BC_DIRICHLET_EQ) return false;
-        if (!in.initialised) continue;
-        cells += static_cast<long long>(in.nx) * in.ny;
-        ++count;
-    }
-    return count > 0 && cells >= count * (b->storage == LBM_F32 ? 36000 : 16000);
+    for (const auto& kv : b->insts)
+        if (kv.second.bc != LBM_BC_DIRICHLET_EQ) return false;
+    return true;
+}
+
+// Cells of the initialised instances: of the lattices, of the marching walks in and outside
+// the rectangles without checks, of the two-step tiles, and instances.
+struct BatchCells {
+    long long lattice = 0, fast = 0, general = 0, tiles = 0, count = 0;
+    size_t largest_launch = 0;  // instances in the largest marching launch
+};
+
+// Whether they are the faster ones, ratio of throughputs to the tile kernels (one variant
+// where none is named):
+//  - FP32: the walks, weighed by what their cells cost (5.8 ps in the rectangles, 10 outside,
+//    10.8 a tile's), must cost less than the tiles: 64 of 400^2 1.45, 32 of 1000 x 64 1.31, 100 of
+//    64^2 with one 2048^2 1.20, 16 of 190^2 0.98, 32 of 64 x 1000 (two strips of 60 columns
+//    each) 0.86.  Small instances leave a warp little but edges and constants that change
+//    with every block: 64 of 64-128 0.91, 32 of 64-256 0.91, hence 36,000 cells on average.  And
+//    there must be enough to fill the device, or a large lattice: 8 of 256^2 0.52 million cells 1.22, but 8 of 190^2 0.83, 4 of 256^2 0.95, 4 of
+//    320^2 of four variants 0.90; single ones of 400^2 1.37, 320^2 0.98.
+//  - 16-bit: a launch of many small instances loses to the constants that change from block
+//    to block: 64 of 128^2 0.63, 32 of 64 x 1000 0.53, 64 of 256^2 0.95, 600 x 100 0.92, but 16 of
+//    256^2 1.14 and 64 of 256^2 of five variants (launches of 13) 1.37.  Launches of more than
+//    23 must gain by their cells too (50 of 64^2 with one 2048^2 1.32; 400 with one 4096^2
+//    0.90), and instances of 20,000 cells on average are needed (16 of 128^2 0.91, 160^2 1.06).
+bool march_pays(const lbm_batch_ctx* b, const BatchCells& c) {
+    if (b->storage == LBM_F32)
+        return c.lattice >= 36000 * c.count && 0.58 * c.fast + c.general <= c.tiles &&
+               (c.lattice >= 600000 || c.lattice >= 150000 * c.count);
+    return c.lattice >= 20000 * c.count &&
+           (c.largest_launch < 24 || 0.64 * c.fast + 2.1 * c.general <= c.tiles);
 }
 
 // Group the initialised instances for marching launches.
 void build_march_groups(lbm_batch_ctx* b) {
     b->march_groups.clear();
-    b->march = march_pays(b);
+    b->march = march_serves(b);
     if (!b->march) return;
     const int nl = march_levels(b);
+    BatchCells cells;
     std::map<int, std::vector<int>> by_variant;
     for (const auto& kv : b->insts)
         if (kv.second.initialised) by_variant[kv.second.variant].push_back(kv.first);
@@ -985,6 +1004,7 @@ void build_march_groups(lbm_batch_ctx* b) {
             lbm_batch_ctx::MarchGroup g;
             g.variant = variant;
             for (size_t i = q; i < ids.size(); i += groups) g.ids.push_back(ids[i]);
+            cells.largest_launch = std::max(cells.largest_launch, g.ids.size());
             for (const int id : g.ids) {
                 const Instance& in = b->insts.at(id);
                 lbm::MarchItem it{};
@@ -996,16 +1016,29 @@ void build_march_groups(lbm_batch_ctx* b) {
                 it.pitch = static_cast<int>(in.geo.pitch);
                 it.plane = static_cast<unsigned>(in.geo.plane);
                 it.grid = lbm::march_rectangle(in.geo, it.k, in.variant, nl);
+                const long long fast = lbm::march_fast_cells(it.grid, nl);
+                cells.lattice += static_cast<long long>(in.nx) * in.ny;
+                cells.fast += fast;
+                cells.general += lbm::march_cells(it.grid, in.ny, nl) - fast;
+                cells.tiles += static_cast<long long>((in.nx + lbm::kTbW - 1) / lbm::kTbW) *
+                               ((in.ny + lbm::kTbH - 1) / lbm::kTbH) * lbm::kTbW * lbm::kTbH;
+                ++cells.count;
                 g.items.push_back(it);
             }
-            lbm::march_segment(nl, b->sms, [&](int seg) {
-                long long blocks = 0;
-                for (auto& it : g.items) blocks += lbm::march_cut(it.grid, it.ny, seg);
-                return blocks;
-            });
             b->march_groups.push_back(std::move(g));
         }
     }
+    b->march = cells.count > 0 && march_pays(b, cells);
+    if (!b->march) {
+        b->march_groups.clear();
+        return;
+    }
+    for (auto& g : b->march_groups)
+        lbm::march_segment(nl, b->sms, [&](int seg) {
+            long long blocks = 0;
+            for (auto& it : g.items) blocks += lbm::march_cut(it.grid, it.ny, seg);
+            return blocks;
+        });
 }
 
 // Advance every active instance by the d steps of a marching launch from global step s0;

@@ -89,3 +89,50 @@ def test_the_choice_follows_the_layer_until_a_kernel_is_named():
         lat.set_sponge("III", thick, thick)
         lat.step(5)
         np.testing.assert_array_equal(got, lat.get_state()[0])
+
+
+V5 = ["none", "I", "II", "III", "viscous"]
+
+
+# (instances as (count, shape), storage, variants in turn, marching)
+@pytest.mark.parametrize("shapes,storage,variants,marching", [
+    ([(4, (400, 390))], "f32", ["II"], True), ([(1, (700, 690))], "f32", ["I"], True),
+    ([(16, (256, 250))], "f32", V5, True),
+    ([(25, (64, 64)), (1, (1024, 1000))], "f32", ["II"], True),
+    ([(4, (256, 256))], "f32", ["II"], False), ([(8, (190, 190))], "f32", ["III"], False),
+    ([(32, (64, 1000))], "f32", ["II"], False), ([(64, (100, 100))], "f32", ["I"], False),
+    ([(16, (256, 250))], "f16dev", ["II"], True), ([(2, (160, 170))], "bf16dev", ["II"], True),
+    ([(40, (200, 190))], "bf16dev", V5, True),
+    ([(30, (64, 64)), (1, (2048, 1500))], "f16dev", ["none"], True),
+    ([(32, (64, 1000))], "f16dev", ["III"], False), ([(30, (200, 200))], "bf16dev", ["I"], False),
+    ([(16, (128, 130))], "f16dev", ["II"], False)])
+def test_batches_march_where_it_is_faster(shapes, storage, variants, marching, monkeypatch):
+    from test_gpu_launches import _kernels
+
+    from paper_1203_6350_gb300.batch import Batch
+
+    def fields(expect):
+        with Batch(storage, config={"cells": 2, "steps_per_launch": 2, "tile": (64, 16)}) as b:
+            ids = []
+            for count, (nx, ny) in shapes:
+                for _ in range(count):
+                    v = variants[len(ids) % len(variants)]
+                    w = 0 if v == "none" else 20
+                    i = b.add(nx, ny, 1000, s=1.6, u0=(0.04, -0.02), variant=v,
+                              chi_x=_ramp(nx, w), chi_y=_ramp(ny, w))
+                    b.init_pulse(i, 1e-3, 6.0, 0.4 * nx, 0.6 * ny)
+                    ids.append(i)
+            b.step(1)
+            for _ in range(2):  # (the first trace of a process may hold nothing)
+                names = _kernels(lambda: b.step(12))
+            if any("batch" in n for n in names):
+                assert any("march_batch" in n for n in names) == expect
+            for n in (4, 7, 35):
+                b.step(n)
+            return [b.moments(i) for i in ids]
+
+    monkeypatch.delenv("LBM_BATCH_TMA", raising=False)
+    got = fields(marching)
+    monkeypatch.setenv("LBM_BATCH_TMA", "1")
+    for a, b in zip(got, fields(False)):
+        np.testing.assert_array_equal(a, b)
