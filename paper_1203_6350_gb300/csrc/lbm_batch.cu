@@ -1547,7 +1547,9 @@ int lbm_batch_step(lbm_batch b, int nsteps) {
         ++launch_off;
         nsteps -= d;
     }
-    if (launch_off > 0) {
+    // a graph reads the device's counters; single launches take the offsets to them
+    const bool graph = cs == cudaStreamCaptureStatusNone && nsteps >= kBatchChunk;
+    if (graph && launch_off > 0) {
         lbm::advance_counters_kernel<<<1, 1, 0, b->stream>>>(b->d_counters, step_off, launch_off);
         e = cudaGetLastError();
         if (e != cudaSuccess) return bfail(b, LBM_ERR_CUDA, std::string("batch advance: ") + cudaGetErrorString(e));
@@ -1555,7 +1557,7 @@ int lbm_batch_step(lbm_batch b, int nsteps) {
         b->launches += launch_off;
         step_off = launch_off = 0;
     }
-    if (cs == cudaStreamCaptureStatusNone && nsteps >= kBatchChunk) {
+    if (graph) {
         e = ensure_batch_graph(b);
         if (e != cudaSuccess) return bfail(b, LBM_ERR_CUDA, std::string("batch graph: ") + cudaGetErrorString(e));
         const int n = kBatchChunk / b->spl;

@@ -136,3 +136,22 @@ def test_batches_march_where_it_is_faster(shapes, storage, variants, marching, m
     monkeypatch.setenv("LBM_BATCH_TMA", "1")
     for a, b in zip(got, fields(False)):
         np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("storage,steps", [("f32", 4), ("f32", 8), ("f16dev", 5)])
+def test_a_short_call_moves_the_clock_once(storage, steps):
+    """The steps that marching launches leave over read the clock at an offset."""
+    from test_gpu_launches import _kernels
+
+    from paper_1203_6350_gb300.batch import Batch
+
+    with Batch(storage, config={"cells": 2, "steps_per_launch": 2, "tile": (64, 16)}) as b:
+        i = b.add(700, 690, 1000, s=1.6)
+        b.init_pulse(i, 1e-3, 6.0, 300.0, 300.0)
+        b.step(1)
+        for _ in range(2):  # (the first trace of a process may hold nothing)
+            names = _kernels(lambda: b.step(steps))
+        if any("batch" in n for n in names):
+            assert any("march_batch" in n for n in names)
+            assert sum("advance_counters" in n for n in names) == 1
+        assert b.time(i) == 1 + 2 * steps
