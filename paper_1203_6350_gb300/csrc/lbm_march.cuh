@@ -157,28 +157,18 @@ __device__ __forceinline__ void march(const T* __restrict__ src, T* __restrict__
                     y = wrapped(y, ny);
                     const int cw = column[i];
                     const char* row = from[i] + static_cast<size_t>(y) * pitch_b;
-                    if (cw + 4 <= nx && (cw & 3) == 0) {
+                    // (16-bit rows are a multiple of 4 long, so every chunk is whole and aligned)
+                    if (ES == 2 || (cw + 4 <= nx && (cw & 3) == 0)) {
                         asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(to),
                                      "l"(row), "n"(4 * ES)
                                      : "memory");
                     } else {  // a chunk across the seam, or shifted by a row length not a multiple of 4
-                        auto past = [&](int e) {  // bytes from the chunk's start to its element e
-                            int d = cw + e;
-                            if (d >= nx) d = nx >= 4 ? d - nx : d % nx;
-                            return (d - cw) * ES;
-                        };
-                        if (ES == 4 || (nx & 1) == 0) {  // in words of four bytes
 #pragma unroll
-                            for (int e = 0; e < 4; e += 4 / ES)
-                                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(
-                                                 to + e * ES),
-                                             "l"(row + past(e))
-                                             : "memory");
-                        } else {
-                            T* d = ring + (slot_in * kMarchStage + q) * 4;
-#pragma unroll
-                            for (int e = 0; e < 4; ++e)
-                                d[e] = __ldg(reinterpret_cast<const T*>(row + past(e)));
+                        for (int e = 0; e < 4; ++e) {
+                            const int past = cw + e >= nx ? e - nx : e;  // elements from the chunk's start
+                            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(to + e * ES),
+                                         "l"(row + past * ES)
+                                         : "memory");
                         }
                     }
                 } else {
@@ -375,12 +365,15 @@ __global__ void __launch_bounds__(32, march_per_sm(NL))
 }
 
 // Advance NL steps: src holds time t, dst receives t + NL; pdl as for the one-step
-// kernels.  cudaErrorInvalidValue when the nine planes exceed 32-bit offsets.
+// kernels.  cudaErrorInvalidValue when the nine planes exceed 32-bit offsets, and for periodic
+// rows that the staging does not take: shorter than a chunk, or 16-bit and no multiple of it.
 template <typename T, int BC, int NL, bool RND>
 cudaError_t launch_march_t(const void* src, void* dst, const Geometry& g, const StepConst<F2>& k,
                            const AxisCoef<float>* tx, const AxisCoef<float>* ty, int variant,
                            int seg, cudaStream_t st, int pdl) {
     if (9 * g.plane >= (1ll << 32)) return cudaErrorInvalidValue;
+    if (BC == kPeriodic && (g.nx < 4 || (sizeof(T) == 2 && g.nx % 4 != 0)))
+        return cudaErrorInvalidValue;
     MarchGrid m = march_rectangle(g, k, variant, NL);
     march_cut(m, g.ny, seg);
     cudaLaunchConfig_t cfg = {};
