@@ -440,9 +440,59 @@ def run_native(args):
             "compensated_arithmetic": comp,
             "decay_exponent": decay,
         }
-        print(json.dumps(line), flush=True)
+        # the whole record beside the line, whose reader may take the last few kilobytes only
+        print(json.dumps(finite(line)), file=sys.stderr, flush=True)
+        print(json.dumps(summary_line(line)), flush=True)
     if world > 1:
         torch.distributed.destroy_process_group()
+
+
+def finite(v):
+    """v with null in the place of every number that JSON has no form for."""
+    if isinstance(v, dict):
+        return {k: finite(x) for k, x in v.items()}
+    if isinstance(v, (list, tuple)):
+        return [finite(x) for x in v]
+    return None if isinstance(v, float) and not math.isfinite(v) else v
+
+
+def summary_line(record: dict) -> dict:
+    """The line of a run: the record's headline as it is, and of each leg its main
+    figures."""
+    legs = {"roofline_sweep", "line_source", "stability_map", "d3q15", "batched", "serving",
+            "parity", "compensated_arithmetic", "decay_exponent", "divergent_solves"}
+    out = {k: v for k, v in record.items() if k not in legs}
+    for k in ("roofline", "roofline_large"):
+        if out.get(k):
+            out[k] = {q: out[k][q] for q in ("bound", "achieved", "peak", "unit", "frac", "kernel",
+                                             "steps_per_launch", "avg_launch_us", "mlups",
+                                             "bytes_per_launch") if q in out[k]}
+    if out.get("cpu_baseline"):
+        out["cpu_baseline"] = {q: v for q, v in out["cpu_baseline"].items() if q != "timings"}
+
+    def leg(name, *path):
+        v = record.get(name)
+        for q in path:
+            v = v.get(q) if isinstance(v, dict) else None
+        return v
+
+    parity = record.get("parity") or {}
+    out["legs"] = {k: v for k, v in {
+        "divergent_solves": sorted(record.get("divergent_solves") or {}),
+        "line_source_mlups": leg("line_source", "mlups"),
+        "stability_map_cases_per_s": leg("stability_map", "f32", "cases_per_s"),
+        "d3q15_256_mlups": leg("d3q15", "f32", "mlups"),
+        "batched_mlups": leg("batched", "mlups"),
+        "served_solves_per_s": leg("serving", "served", "solves_per_s"),
+        "served_p99_s": leg("serving", "served", "p99_s"),
+        "serving_speedup": leg("serving", "solves_per_s_speedup_vs_plain"),
+        "parity_cases": len(parity["cases"]) if "cases" in parity else None,
+        "parity_missed": len(parity["missed"]) if "missed" in parity else None,
+        "compensated_mlups": leg("compensated_arithmetic", "1024x1024 Mach 0.2",
+                                 "compensated_mlups"),
+        "decay_slope": leg("decay_exponent", "rest", "gpu_slope"),
+    }.items() if v not in (None, [])}
+    return finite(out)
 
 
 def with_warn(fn):
