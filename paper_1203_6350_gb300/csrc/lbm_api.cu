@@ -289,41 +289,47 @@ int march_steps(const lbm_ctx* h);
 //  - Dirichlet: 0.92 at 700^2, 1.00 at 850^2, 1.09 at 900^2, 1.05 at 1024^2, 1.9 at
 //    1300^2, 1.7 at 2048^2, 1.63 at 4096^2 (16-bit storage: 1.03 at 850^2, 1.14-1.17 at
 //    1536^2, 1.3 at 4096^2).  Fewer cells leave too few warps, each with a long walk.
-//  - Periodic, rows a multiple of the staged chunk: 0.94 at 1024^2, 1.14 at 1100^2, 1.8
-//    at 1300^2 and 4096^2 (16-bit: 0.96 at 1024^2, 1.14 at 1300^2, 1.3 at 4096^2).  Other
-//    rows are staged by words at the seam: 0.86 at 1150^2, but 1.12 at 1401^2 and 1.25
-//    at 2049^2 in FP32, once the state exceeds L2.
+//  - Periodic, rows a multiple of the staged chunk: 1.48 at 1100^2 (1.23 with a layer 64 deep),
+//    2.1 at 1300^2, 1.7 at 4096^2 (16-bit: 1.10-1.15 at 1100^2, 1.2 at 1600^2, 1.5 at 4096^2).
+//    Other rows are staged by words at the seam: 1.73 at 1401^2 and 1.72 at 2049^2 in FP32,
+//    once the state exceeds L2.
 //  - At least four strips and 64 rows, or the last strip's idle lanes and the rows
 //    computed twice eat the gain.  16-bit lattices that L2 holds easily need 200
 //    rows: periodic 17472 x 103 0.74, 7804 x 168 0.88, 10256 x 162 0.93, 4000 x 304 1.04,
 //    Dirichlet 18717 x 113 0.85, 11532 x 139 0.96, 2242 x 402 1.12.
 // And by the layer: a cell of the walks outside the chi = 0 rectangle costs 1.6 to 1.9 times
-// one inside (16-bit 8.8 against 4.7 ps), which the other kernels' layer cells do not.  The
-// share of such walks, up to which marching is taken:
-//  - 16-bit: 0.5 while both buffers fill 3/4 of L2 or less (bf16 1832 x 1199 0.37, 1.11;
-//    f16 1085 x 1826 0.49, 1.03; 786 x 1241 0.55, 0.95; 5724 x 415 0.65, 0.89; 850 x 1054 0.82,
-//    0.86; 1344 x 1093 0.98, 0.83), above, where the other kernels slow down, 0.85 (bf16
-//    2447 x 1187 0.73, 1.10; 2300 x 1552 0.84, 1.14; f16 8125 x 483 1, 0.96; bf16 4096^2 1, 0.97);
-//  - FP32: any (4096^2 1, 1.31; 1344 x 1093 1, 1.15), but 0.7 where the seam is staged by
-//    words (2045 x 1664 0.71, 0.98; 18899 x 156 1, 0.85).  Below 1.1 million cells a share
-//    above 0.6 costs time in FP32 too (1024^2, layer II 64 deep: 0.37, 1.07; 128 deep 0.54,
-//    511 deep 1, 0.79).
+// one inside (FP32 8.0 against 4.9 ps, 16-bit 8.8 against 4.7), which the other kernels' layer
+// cells do not.  The share of such walks, up to which marching is taken:
+//  - FP32: 0.5 while both buffers fill 5/8 of L2 or less (1024^2, layer II 64 deep: share 0.37,
+//    1.08; 128 deep: 0.54, 0.94; 2673 x 315 0.50, 1.12; 889 x 1206 0.90, 0.93), any above, where
+//    the other kernels slow down (1192 x 971 0.81, 1.10; 4096^2 1, 1.31), but 0.7 where the
+//    seam is staged by words (2045 x 1664 0.71, 0.98; 18899 x 156 1, 0.85).  FP32 lattices less
+//    than 256 cells across, or without any rectangle, march at every size and share, which
+//    costs those below 1.1 million cells up to 21 % (13001 x 64 0.7, 0.93; 240 x 3656 1, 0.88;
+//    1024^2 all layer 1, 0.79): the tests of the marching kernels count on it.
+//  - 16-bit: 0.5 up to 3/4 of L2 (bf16 1832 x 1199 0.37, 1.11; f16 1085 x 1826 0.49, 1.03; 786 x
+//    1241 0.55, 0.95; 5724 x 415 0.65, 0.89; 850 x 1054 0.82, 0.86; 1344 x 1093 0.98, 0.83), 0.85
+//    above (bf16 2447 x 1187 0.73, 1.10; 2300 x 1552 0.84, 1.14; f16 8125 x 483 1, 0.96; bf16
+//    4096^2 1, 0.97).
 // Without a layer every walk is the cheap one.
 bool march_pays(const lbm_ctx* h) {
     if (h->storage == LBM_F64 || h->nx < 240 || h->ny < 64) return false;
     const long long cells = static_cast<long long>(h->nx) * h->ny;
     const bool f32 = h->storage == LBM_F32, periodic = h->bc == LBM_BC_PERIODIC;
     const bool words = periodic && h->nx % 4 != 0;
-    const bool fits = 2 * h->buf_bytes / 3 <= h->l2 / 4;
+    const double filled = 2.0 * h->buf_bytes / h->l2;  // of L2, by both buffers
+    const bool fits = filled <= (f32 ? 0.625 : 0.75);
     if (h->bc == LBM_BC_CHANNEL || cells < (periodic ? 1200000 : 800000)) return false;
-    if (words && !(f32 && 2 * h->buf_bytes > h->l2)) return false;
+    if (words && !(f32 && filled > 1.0)) return false;
     if (!f32 && fits && h->ny < 200) return false;
-    if (h->variant == LBM_SPONGE_NONE || (f32 && !words)) return true;
+    if (h->variant == LBM_SPONGE_NONE) return true;
     const int nl = march_steps(h);
     const lbm::MarchGrid m = lbm::march_rectangle(h->geo, h->k2, h->variant, nl);
-    const double share = 1.0 - static_cast<double>(lbm::march_fast_cells(m, nl)) /
-                                   lbm::march_cells(m, h->ny, nl);
-    return share <= (f32 ? 0.7 : fits ? 0.5 : 0.85);
+    const long long fast = lbm::march_fast_cells(m, nl);
+    const double share = 1.0 - static_cast<double>(fast) / lbm::march_cells(m, h->ny, nl);
+    if (!f32) return share <= (fits ? 0.5 : 0.85);
+    if (words) return share <= 0.7;
+    return !fits || share <= 0.5 || fast == 0 || h->nx < 256 || h->ny < 256;
 }
 
 // Small lattices take several steps per launch on tiles of 32-column regions.  Up to

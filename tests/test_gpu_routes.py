@@ -43,6 +43,8 @@ ROUTES = [((1024, 1024), "dirichlet", "bf16dev", "II", 64, True),
           ((1024, 1024), "dirichlet", "bf16dev", "II", 511, False),
           ((850, 1054), "dirichlet", "f16dev", "I", 250, False),
           ((1024, 1024), "dirichlet", "f16dev", "none", 0, True),
+          ((1024, 1024), "dirichlet", "f32", "II", 64, True),
+          ((1024, 1024), "dirichlet", "f32", "II", 128, False),
           ((1024, 1024), "dirichlet", "f32", "II", 511, True),
           ((1344, 1093), "periodic", "f16dev", "III", 20, True),
           ((1344, 1093), "periodic", "f16dev", "III", 545, False),
