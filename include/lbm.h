@@ -149,11 +149,11 @@ int lbm_init_pulse(lbm_handle h, double eps, double half_width, double x0, doubl
 
 /* Advance nsteps >= 0 time steps by fused kernels (pull-stream, moments, rho*
  * and j*, MRT relaxation, damping term, back-transform, store), asynchronous
- * on the handle's stream.  Large lattices (about 900 x 900 cells and more)
- * take groups of two or three steps per launch, by warps that march down the
- * lattice with the time levels between in registers, and small ones (up to
- * 226 x 226 cells) up to six, on tiles in shared memory; the results are those of
- * the launches that lbm_set_steps_per_launch describes, bit for bit, and
+ * on the handle's stream.  Large lattices (about 900 x 900 cells and more, where
+ * the layer leaves enough of them in the bulk) take groups of two or three steps per
+ * launch, by warps that march down the lattice with the time levels between in
+ * registers, and small ones (up to 226 x 226 cells, unless they are very thin) up to six,
+ * on tiles in shared memory; the results are those of the launches that lbm_set_steps_per_launch describes, bit for bit, and
  * lbm_set_steps_per_launch or lbm_set_tma_staging (or their environment
  * variables) select those launches instead.
  *
@@ -386,10 +386,11 @@ int lbm_batch_cells_per_thread(lbm_batch b);
  * takes that one step.  Needs two cells per thread
  * (lbm_batch_set_cells_per_thread(b, 1) switches it back to 1).  Default 1.
  * With 2, batches of Dirichlet instances of some size (36,000 cells on average,
- * 16,000 with 16-bit storage) take two (FP32: three) steps per launch by the
- * marching kernels of lbm_step, with the same results, as long as every active
- * instance has that many left; the environment variable LBM_BATCH_TMA (either
- * value) keeps to the tiles.
+ * 20,000 with 16-bit storage, and enough of them or of their bulk) take two (FP32:
+ * three) steps per launch by the marching kernels of lbm_step, with the same results, as
+ * long as every active instance has that many left; the environment variable
+ * LBM_BATCH_TMA (either value) keeps to the tiles, and so does a batch once one of its
+ * steps has been captured into a graph, whose replays the host does not see.
  * LBM_ERR_ARG for any other value or an unsupported 2.  Waits for the
  * batch's stream. */
 int lbm_batch_set_steps_per_launch(lbm_batch b, int steps);

@@ -193,7 +193,7 @@ __device__ __forceinline__ void cell_moments(const PlanePtrs<T>& src, const Geom
 // rho', u of every cell.  States held in FP32 or less: one reciprocal per cell (two FP64
 // instructions) in place of two divisions, and no conversion instructions: eleven FP64
 // instructions per cell, which bound it.  4096^2 FP32, 36 + 24 B per cell: 1143 us
-// with divisions, 472 us now (2.1 TB/s; floor 150 us), the same bits.
+// with divisions, 409 us now (2.5 TB/s; floor 150 us), the same bits.
 template <typename T, int BC>
 __global__ void __launch_bounds__(256)
     moments_kernel(PlanePtrs<T> src, Geometry g, BaseState b, double* rho_dev, double* ux,

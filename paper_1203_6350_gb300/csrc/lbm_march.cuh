@@ -30,9 +30,10 @@
 // the rectangle of the rest.  In that rectangle no cell touches the lattice's
 // edge or the layer (chi = 0) and nothing is checked.
 //
-// What bounds it: the FMA pipe and the issue slots (three levels at 4096^2: FMA 69 %
-// and issue 64 % busy; a packed FMA takes the pipe for two cycles, so 95 of them per
-// pair and level cap the chip at 391 GLUPS).
+// What bounds it: HBM and the FMA pipe together (three levels at 4096^2: DRAM at 0.84 of
+// its measured rate, the FMA pipe 65 % and the issue slots 59 % busy; a packed FMA takes
+// the pipe for two cycles, so 95 of them per pair and level cap the chip at 391 GLUPS),
+// and below 1.5 million cells the four rows that each short segment walks twice.
 // It moves 24 B (FP32, three levels) or 18 B (16-bit, two) per cell-step to and from
 // HBM.  Measured against the kernels it replaces, GLUPS, FP32 1024^2 / 2048^2 /
 // 4096^2 / 8192^2: 146 / 129 / 148 / 150 before, 153 / 219 / 242 / 259 with it; BF16
